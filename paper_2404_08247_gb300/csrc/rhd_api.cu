@@ -334,6 +334,8 @@ void rhd::fill_geometry(const rhd_params* p, Geometry& g, Physics& ph) {
   ph.kappa_P_ratio = p->kappa_P_ratio;
   ph.kappa_F_ratio = p->kappa_F_ratio;
   ph.reconstruction = p->reconstruction;
+  ph.inv_cv_spec = 1.0 / ph.cv_spec;
+  fill_start(ph.start, p->c, p->chat, p->a_rad, ph.cv_spec, p->newton_rtol, p->outer_rtol);
 }
 
 static void release(rhd_ctx* c) {

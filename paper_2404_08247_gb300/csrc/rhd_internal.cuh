@@ -11,6 +11,7 @@
 #include <stdint.h>
 
 #include "rhd.h"
+#include "rhd_start.cuh"
 
 namespace rhd {
 
@@ -83,6 +84,8 @@ struct Physics {
   double kappa_P_ratio;    // chi_0P / chi_0E
   double kappa_F_ratio;    // chi_0F / chi_0E
   int reconstruction;      // rhd_recon
+  double inv_cv_spec;      // 1/cv_spec
+  StartConsts start;       // constants of pair_start
 };
 
 struct StageArgs {
@@ -131,12 +134,14 @@ inline void slots_of(P* out, P base, int n) {
 // with the integer pipe doing what it can:
 //  * non-negative, non-NaN doubles order like their IEEE bit patterns as
 //    signed 64-bit integers, so their compares and minima are integer ops;
-//  * rcp_pos / rsqrt_pos: 1/x and 1/sqrt(x) for x > 0 by Newton-Raphson
-//    iteration (r <- r + r (1 - x r); y <- y + y (1/2 - x y^2 / 2), each step
-//    doubling the correct bits; e.g. P. Markstein, IBM J. Res. Dev. 34 (1990))
+//  * rcp_pos / rsqrt_pos / sqrt_pos: 1/x, 1/sqrt(x) and sqrt(x) for x > 0
 //    from a single-precision seed whose exponent is rebiased with integer
-//    arithmetic: two steps from a 2^-22 seed leave ~1 ulp (the IEEE operation
-//    is used outside the single-precision exponent range).
+//    arithmetic (relative error below 2^-21) and the binomial series in its
+//    residual e up to the second order: r (1 + e + e^2) with e = 1 - x r, and
+//    y (1 + e/2 + 3 e^2/8) with e = 1 - x y^2.  The third order, left out, is
+//    below 2^-63.  3 and 5 FP64 operations, where two Newton steps (quadratic)
+//    take 4 and 7; within 1 ulp.  The IEEE operation is used outside the
+//    single-precision exponent range.
 constexpr long long kMag = 0x7fffffffffffffffll;
 constexpr long long kInfBits = 0x7ff0000000000000ll;
 
@@ -167,22 +172,45 @@ __device__ __forceinline__ float seed_float(double x) {
 __device__ __forceinline__ double seed_double(float f) {
   return __longlong_as_double(((long long)__float_as_int(f) + (896ll << 23)) << 29);
 }
+// One rounding each, never contracted with a neighbour: a cell's solve gives the
+// same bits in every kernel that runs it.
+__device__ __forceinline__ double mul(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ double add(double a, double b) { return __dadd_rn(a, b); }
+__device__ __forceinline__ double sub(double a, double b) { return __dadd_rn(a, -b); }
+__device__ __forceinline__ double dot3(const double a[3], const double b[3]) {
+  return fma(a[2], b[2], fma(a[1], b[1], mul(a[0], b[0])));
+}
+
+// 1/x to about 2^-21 for x > 0, off the FP64 pipe (outside the single-precision
+// exponent range: the division)
+__device__ __forceinline__ double rcp_approx(double x) {
+  return seed_range(x) ? seed_double(__fdividef(1.0f, seed_float(x))) : 1.0 / x;
+}
 __device__ __forceinline__ double rcp_pos(double x) {
   if (!seed_range(x)) return 1.0 / x;
-  double r = seed_double(__fdividef(1.0f, seed_float(x)));
-  double e = fma(-x, r, 1.0);
-  r = fma(r, e, r);
-  e = fma(-x, r, 1.0);
-  return fma(r, e, r);
+  const double r = seed_double(__fdividef(1.0f, seed_float(x)));
+  const double e = fma(-x, r, 1.0);
+  return fma(r, fma(e, e, e), r);
+}
+// the series' relative correction to the seed y of 1/sqrt(x), and t = x y
+__device__ __forceinline__ double rsqrt_corr(double x, double y, double& t) {
+  t = mul(x, y);
+  const double e = fma(-t, y, 1.0);
+  return mul(e, fma(0.375, e, 0.5));
 }
 __device__ __forceinline__ double rsqrt_pos(double x) {
   if (!seed_range(x)) return 1.0 / sqrt(x);
-  double y = seed_double(rsqrtf(seed_float(x)));
-  double h = 0.5 * x;
-  double e = fma(-h * y, y, 0.5);
-  y = fma(y, e, y);
-  e = fma(-h * y, y, 0.5);
-  return fma(y, e, y);
+  const double y = seed_double(rsqrtf(seed_float(x)));
+  double t;
+  const double q = rsqrt_corr(x, y, t);
+  return fma(y, q, y);
+}
+__device__ __forceinline__ double sqrt_pos(double x) {
+  if (!seed_range(x)) return sqrt(x);
+  const double y = seed_double(rsqrtf(seed_float(x)));
+  double t;
+  const double q = rsqrt_corr(x, y, t);
+  return fma(t, q, t);
 }
 
 // ---------------------------------------------------------------- limiter
@@ -373,16 +401,15 @@ __device__ __forceinline__ void m1_coeffs(R E, const R Ft[3], R& ha, R& hb) {
 template <>
 __device__ __forceinline__ void m1_coeffs<double>(double E, const double Ft[3], double& ha,
                                                   double& hb) {
-  double F2 = Ft[0] * Ft[0] + Ft[1] * Ft[1] + Ft[2] * Ft[2];
-  double E2 = E * E;
+  const double F2 = dot3(Ft, Ft);
+  const double E2 = mul(E, E);
   if (lt_nn(E2, F2)) {
     ha = 0.0;
-    hb = E * rcp_pos(F2);
+    hb = mul(E, rcp_pos(F2));
   } else {
-    double x = 4.0 * E2 - 3.0 * F2;
-    double s = x * rsqrt_pos(x);
-    ha = (s - E) * (1.0 / 3.0);
-    hb = 3.0 * rcp_pos(2.0 * E + s);
+    const double s = sqrt_pos(fma(-3.0, F2, mul(4.0, E2)));
+    ha = mul(sub(s, E), 1.0 / 3.0);
+    hb = mul(3.0, rcp_pos(fma(2.0, E, s)));
   }
 }
 
@@ -597,176 +624,215 @@ __device__ __forceinline__ bool quartic_start(double a4, double rhs, double T0, 
 //   r1 = k g F_R = k g (aT^4 - E(t) - R) + k v.F/c^2 - R
 //   J  = [[1, c/chat], [g k 4 a T^3 / C_v, -g (1 + k)]]
 // converged when |r0| < eps E_tot and (c/chat)|r1| <= eps E_tot k g,
-// E_tot = Egas(t) + (c/chat) E(t).  The first pass starts from quartic_start
-// (constant chi) or from (Egas(t), 0) (chi ~ T^p, whose J10 gains the term of
-// the T-dependence of k).
+// E_tot = Egas(t) + (c/chat) E(t).  The iteration starts from pair_start's
+// near-converged (R, F); if that gives up, or the iteration fails from there,
+// from quartic_start and the explicit F, and with chi ~ T^p (whose J10 gains
+// the term of the T-dependence of k) from (Egas(t), 0).
 // Energy closure: E = E(t) - (chat/c)(Egas - Egas(t)).
 // Outer stage: eq. (numF2) (order 2) or (numF1) (order 1) for F with P from
 // the new E and the previous outer flux, momentum m = m(t) - (F - F(t))/(c chat),
 // repeated until Q = k[(g - 1)(aT^4 - E) + v.F/c^2] settles: its change is at
 // most outer_rtol times |Q|, |R| or the magnitude of its terms.
-// MIXED: the Newton step's reciprocal of the Jacobian determinant is taken in
-// single precision (a step off by 1e-7 only slows the last iteration by that
-// factor); residuals, the state, the closure of the exchange term v.P and
-// every update stay double, so the solve meets the double-precision
-// convergence tests (inner and outer) and conserves to rounding.
+// MIXED: the reciprocal of the Jacobian determinant is a seed of 2^-21 (a step
+// off by that factor only slows the last update); residuals, the state, the
+// closure of the exchange term v.P and every update stay double, so the solve
+// meets the double-precision convergence tests (inner and outer) and conserves
+// to rounding.
 // GEN: compiled with the temperature-dependent opacity; the default physics
 // (constant chi) uses the GEN = false copy, free of that branch.
+constexpr double kNear = 1e4;  // in units of the Newton tolerance
+
 template <bool MIXED, bool GEN>
 __device__ __forceinline__ int local_solve(const Physics& ph, double tdt, double rho,
                                            double chi, double y[8], int& nn, int& no) {
   nn = 0;
   no = 0;
   if (chi == 0.0) return RHD_OK;
-  const double Cv = rho * ph.cv_spec;
-  const double inv_Cv = rcp_pos(Cv);
+  const double Cv = mul(rho, ph.cv_spec);
   const double inv_rho = rcp_pos(rho);
+  const double inv_Cv = mul(inv_rho, ph.inv_cv_spec);
   const double cr = ph.c_over_chat;
   const double a = ph.a_rad;
+  const bool order2 = ph.vc_order == 2;
   const double Eg0 = y[0], E0 = y[4];
-  const double Etot = Eg0 + cr * E0;
+  const double Etot = fma(cr, E0, Eg0);
   // k = chat chi theta dt; with a temperature-dependent opacity chi is taken
   // at the current Newton iterate (the paper's chi carry the superscript
   // (t+1)) and held fixed in the Jacobian
   const bool vary = GEN && ph.kappa_T_exp != 0.0;
-  const double k0 = ph.chat * chi * tdt;
+  const double k0 = mul(mul(ph.chat, chi), tdt);
   double k = k0;
-  const double tolG = ph.newton_rtol * Etot;
-  double Eg = Eg0, R = 0.0, E = E0;
-  double m[3] = {y[1], y[2], y[3]};
+  const double tolG = mul(ph.newton_rtol, Etot);
+  double Eg = Eg0, R = 0.0;
   double F[3] = {y[5], y[6], y[7]};
-
-  // v, beta^2, g, v.F/c^2 and the kinetic energy of the frozen (m, F)
-  double v[3] = {m[0] * inv_rho, m[1] * inv_rho, m[2] * inv_rho};
-  double beta2 = (v[0] * v[0] + v[1] * v[1] + v[2] * v[2]) * ph.inv_c2;
-  double g = (ph.vc_order == 2) ? 1.0 + 0.5 * beta2 : 1.0;
-  double w = (v[0] * F[0] + v[1] * F[1] + v[2] * F[2]) * ph.inv_c2;
-  double Ekin = 0.5 * (m[0] * v[0] + m[1] * v[1] + m[2] * v[2]);
+  double v[3] = {mul(y[1], inv_rho), mul(y[2], inv_rho), mul(y[3], inv_rho)};
 
   // With a temperature-dependent opacity the iteration starts from
   // (Egas(t), 0) like the oracle's: the exact Jacobian below converges
   // quadratically from there, and a common start keeps the two solves on
   // the same iterates near a Marshak front, where the stopping point's
   // rounding is amplified.
-  if (!vary) {
-    double T0 = (Eg0 - Ekin) * inv_Cv;
-    if (pos_finite(T0)) {
-      double kg = k * g;
-      double inv1 = rcp_pos(1.0 + kg);
-      double a4 = cr * kg * a * inv1 * inv_Cv;
-      double rhs = T0 + cr * k * (g * E0 - w) * inv1 * inv_Cv;
-      double Tg;
-      if (pos_finite(rhs) && quartic_start(a4, rhs, T0, Tg)) {
-        Eg = Cv * Tg + Ekin;
-        R = -ph.chat_over_c * (Eg - Eg0);
-      }
+  WarmStart W;
+  W.lag = 0.0;
+  bool warm = !vary && ph.start.ok != 0 &&
+              pair_start(ph.start, ph.closure == RHD_CLOSURE_M1, order2, rho, k0, Etot, y, v,
+                         ph.newton_max, ph.outer_max, W, nn, no);
+  bool settle = warm;  // the first double-precision pass from the warm start
+  if (warm) {
+    R = W.R;
+    Eg = fma(-cr, R, Eg0);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      F[i] = W.F[i];
+      v[i] = mul(fma(-sub(F[i], y[5 + i]), ph.inv_cchat, y[1 + i]), inv_rho);
     }
   }
 
-  for (int outer = 0; outer < ph.outer_max; ++outer) {
-    no = outer + 1;
-    double kg = k * g;
-    double kw = k * w;
-    double c4 = 4.0 * kg * a * inv_Cv;  // J10 / T^3
-    double gpk = g * (1.0 + k);
-    double tolRg = tolG * k * g;
-
-    bool conv = false;
-    double aT4 = 0.0;
-    for (int it = 0;; ++it) {
-      double T = (Eg - Ekin) * inv_Cv;
-      if (!pos_finite(T) || !finite_bits(R)) return RHD_ERR_NONPHYSICAL;
-      if (vary) {
-        k = k0 * pow(T * ph.inv_kappa_T_ref, ph.kappa_T_exp);
-        kg = k * g;
-        kw = k * w;
-        c4 = 4.0 * kg * a * inv_Cv;
-        gpk = g * (1.0 + k);
-        tolRg = tolG * k * g;
+  for (;;) {  // from the warm start; from the cold one if that fails
+    if (!warm) {
+      nn = 0;
+      no = 0;
+      Eg = Eg0;
+      R = 0.0;
+#pragma unroll
+      for (int i = 0; i < 3; ++i) {
+        F[i] = y[5 + i];
+        v[i] = mul(y[1 + i], inv_rho);
       }
-      double T2 = T * T;
-      aT4 = a * T2 * T2;
-      double r0 = (Eg - Eg0) + cr * R;
-      double r1 = kg * (aT4 - E0 - R) + (kw - R);
-      if (lt_nn(fabs(r0), tolG) && le_nn(cr * fabs(r1), tolRg)) {
-        conv = true;
+      const double v2 = dot3(v, v);
+      const double Ekin = mul(mul(0.5, rho), v2);
+      const double T0 = mul(sub(Eg0, Ekin), inv_Cv);
+      if (!vary && pos_finite(T0)) {
+        const double kg = order2 ? fma(k, mul(0.5, mul(v2, ph.inv_c2)), k) : k;
+        const double w = mul(dot3(v, F), ph.inv_c2);
+        const double ck = mul(cr, mul(rcp_pos(add(1.0, kg)), inv_Cv));
+        const double a4 = mul(mul(ck, kg), a);
+        const double rhs = fma(ck, fma(kg, E0, -mul(k, w)), T0);
+        double Tg;
+        if (pos_finite(rhs) && quartic_start(a4, rhs, T0, Tg)) {
+          Eg = fma(Cv, Tg, Ekin);
+          R = mul(-ph.chat_over_c, sub(Eg, Eg0));
+        }
+      }
+    }
+
+    int code = RHD_ERR_OUTER;
+    while (no < ph.outer_max) {
+      ++no;
+      // the frozen (v, F): h = beta^2/2 = g - 1 (0 at order 1), v.F/c^2
+      const double v2 = dot3(v, v);
+      const double h = order2 ? mul(0.5, mul(v2, ph.inv_c2)) : 0.0;
+      const double vF = dot3(v, F);
+      const double w = mul(vF, ph.inv_c2);
+      const double Ekin = mul(mul(0.5, rho), v2);
+      double kg = fma(k, h, k);
+      double kw = mul(k, w);
+
+      double aT4 = 0.0;
+      int inner = RHD_ERR_NEWTON;
+      for (int it = 0;; ++it) {
+        const double T = mul(sub(Eg, Ekin), inv_Cv);
+        if (!pos_finite(T) || !finite_bits(R)) {
+          inner = RHD_ERR_NONPHYSICAL;
+          break;
+        }
+        if (vary) {
+          k = mul(k0, pow(mul(T, ph.inv_kappa_T_ref), ph.kappa_T_exp));
+          kg = fma(k, h, k);
+          kw = mul(k, w);
+        }
+        const double T2 = mul(T, T);
+        aT4 = mul(mul(a, T2), T2);
+        const double r0 = fma(cr, R, sub(Eg, Eg0));
+        const double r1 = fma(kg, sub(sub(aT4, E0), R), sub(kw, R));
+        // a warm start has taken the tests by its lag; its R only has to be
+        // near enough for one update with the determinant's seed (2^-21) to
+        // land at rounding level
+        if (settle && !(lt_nn(fabs(r0), mul(kNear, tolG)) &&
+                        le_nn(mul(cr, fabs(sub(r1, W.lag))), mul(mul(kNear, tolG), kg))))
+          settle = false;
+        const bool conv =
+            settle || (lt_nn(fabs(r0), tolG) && le_nn(mul(cr, fabs(r1)), mul(tolG, kg)));
+        if (conv) inner = RHD_OK;
+        if (conv ? !settle : it >= ph.newton_max) break;
+        const double aT3 = mul(mul(mul(4.0 * a, inv_Cv), T2), T);  // d(a T^4)/dEgas
+        double J10 = mul(kg, aT3);
+        // chi ~ T^p: the R/(k g) term of E(Egas, R) varies with T through k,
+        // which adds p R/(T C_v) to the scaled J10 (exact dE/dEgas; the
+        // paper's J10 holds chi fixed, Sec. 3.3, and converges linearly)
+        if (vary) J10 = add(J10, ph.kappa_T_exp * R / sub(Eg, Ekin));
+        const double gpk = add(add(1.0, h), kg);
+        const double ndet = fma(cr, J10, gpk);  // > 0
+        const double inv_det = settle || MIXED ? rcp_approx(ndet) : rcp_pos(ndet);
+        // settling: the update of the residual beyond the one that the
+        // iteration leaves removes the pairs' rounding from E_gas and R
+        const double r1s = settle ? sub(r1, W.lag) : r1;
+        const double dEg = mul(fma(r0, gpk, mul(cr, r1s)), inv_det);
+        Eg = sub(Eg, dEg);
+        R = fma(-fma(r0, J10, -r1s), inv_det, R);
+        if (settle) {
+          aT4 = fma(-aT3, dEg, aT4);
+          break;
+        }
+        ++nn;
+      }
+      if (inner != RHD_OK) {
+        code = inner;
         break;
       }
-      if (it >= ph.newton_max) break;
-      double J10 = c4 * T2 * T;
-      // chi ~ T^p: the R/(k g) term of E(Egas, R) varies with T through k,
-      // which adds p R/(T C_v) to the scaled J10 (exact dE/dEgas; the
-      // paper's J10 holds chi fixed, Sec. 3.3, and converges linearly)
-      if (vary) J10 += ph.kappa_T_exp * R / (Eg - Ekin);
-      double det = -gpk - cr * J10;  // < 0
-      double inv_det = MIXED ? (double)(1.0f / (float)det) : -rcp_pos(-det);
-      double dEg = (r0 * gpk + cr * r1) * inv_det;
-      double dR = (r0 * J10 - r1) * inv_det;
-      Eg += dEg;
-      R += dR;
-      ++nn;
-    }
-    if (!conv) return RHD_ERR_NEWTON;
 
-    // energy closure; aT4 is that of the converged Egas
-    E = E0 - ph.chat_over_c * (Eg - Eg0);
+      // energy closure; aT4 is that of the converged Egas
+      const double E = fma(-ph.chat_over_c, sub(Eg, Eg0), E0);
 
-    // v_j P_ji of the closure at (E, F): P = ha I + hb Ft Ft^T
-    double vP[3];
-    {
-      double Ft[3] = {F[0] * ph.inv_c, F[1] * ph.inv_c, F[2] * ph.inv_c};
-      if (ph.closure == RHD_CLOSURE_EDDINGTON) {
-        double e3 = E * (1.0 / 3.0);
-        vP[0] = v[0] * e3; vP[1] = v[1] * e3; vP[2] = v[2] * e3;
-      } else {
-        double ha, hb;
-        m1_coeffs(E, Ft, ha, hb);  // the cell flux may exceed the free-streaming limit
-        double t = hb * (v[0] * Ft[0] + v[1] * Ft[1] + v[2] * Ft[2]);
-#pragma unroll
-        for (int i = 0; i < 3; ++i) vP[i] = ha * v[i] + t * Ft[i];
+      // F(t) + k (aT^4 v + v.P) with P = ha I + hb Ft Ft^T at (E, F); the cell
+      // flux may exceed the free-streaming limit
+      const double Ft[3] = {mul(F[0], ph.inv_c), mul(F[1], ph.inv_c), mul(F[2], ph.inv_c)};
+      double ha = mul(E, 1.0 / 3.0), t = 0.0;
+      if (ph.closure == RHD_CLOSURE_M1) {
+        double hb;
+        m1_coeffs(E, Ft, ha, hb);
+        t = mul(hb, mul(vF, ph.inv_c));
       }
-    }
-    double inv_den = rcp_pos(1.0 + kg);
-    double Fn[3], mn[3];
+      const double u = add(aT4, ha);
+      const double inv_den = rcp_pos(add(1.0, kg));
+      const double q = sub(aT4, E);
+      const double Q_old = mul(k, fma(h, q, w));
+      // the updated F, m and v: the next pass freezes these
+      double m[3];
 #pragma unroll
-    for (int i = 0; i < 3; ++i) {
-      Fn[i] = (y[5 + i] + k * (aT4 * v[i] + vP[i])) * inv_den;
-      mn[i] = y[1 + i] - (Fn[i] - y[5 + i]) * ph.inv_cchat;
+      for (int i = 0; i < 3; ++i) {
+        F[i] = mul(fma(k, fma(u, v[i], mul(t, Ft[i])), y[5 + i]), inv_den);
+        m[i] = fma(-sub(F[i], y[5 + i]), ph.inv_cchat, y[1 + i]);
+        v[i] = mul(m[i], inv_rho);
+      }
+      const double hn = order2 ? mul(0.5, mul(dot3(v, v), ph.inv_c2)) : 0.0;
+      const double Q_new = mul(k, fma(hn, q, mul(dot3(v, F), ph.inv_c2)));
+      // |dQ| <= rtol max(|Q_old|, |R|, Q_scale): the three tests of the outer
+      // stop; Q_scale is the magnitude of the terms of Q, the rounding level
+      // of a cancelling v.F
+      const double dQ = fabs(sub(Q_new, Q_old));
+      const double vFa = fma(fabs(v[2]), fabs(F[2]),
+                             fma(fabs(v[1]), fabs(F[1]), mul(fabs(v[0]), fabs(F[0]))));
+      const double Q_scale = mul(k, fma(hn, fabs(q), mul(vFa, ph.inv_c2)));
+      const double big = max_nn(max_nn(fabs(Q_old), fabs(R)), Q_scale);
+      const double tolQ = mul(ph.outer_rtol, big);
+      if (le_nn(dQ, settle ? mul(2.0, tolQ) : tolQ)) {
+        code = pos_finite(E) && finite_bits(F[0]) && finite_bits(F[1]) && finite_bits(F[2])
+                   ? RHD_OK
+                   : RHD_ERR_NONPHYSICAL;
+        if (code == RHD_OK || !warm) {
+          y[0] = Eg;
+          y[1] = m[0]; y[2] = m[1]; y[3] = m[2];
+          y[4] = E;
+          y[5] = F[0]; y[6] = F[1]; y[7] = F[2];
+        }
+        break;
+      }
+      settle = false;
     }
-    double Q_old = k * ((g - 1.0) * (aT4 - E) + w);
-    // the updated v, beta^2, g, v.F/c^2: the next pass freezes these
-    double vn[3] = {mn[0] * inv_rho, mn[1] * inv_rho, mn[2] * inv_rho};
-    double beta2n = (vn[0] * vn[0] + vn[1] * vn[1] + vn[2] * vn[2]) * ph.inv_c2;
-    double gn = (ph.vc_order == 2) ? 1.0 + 0.5 * beta2n : 1.0;
-    double wn = (vn[0] * Fn[0] + vn[1] * Fn[1] + vn[2] * Fn[2]) * ph.inv_c2;
-    double Q_new = k * ((gn - 1.0) * (aT4 - E) + wn);
-    // magnitude of the terms of Q: the rounding level of a cancelling v.F
-    double Q_scale = k * (fabs((gn - 1.0) * (aT4 - E)) +
-                          (fabs(vn[0] * Fn[0]) + fabs(vn[1] * Fn[1]) + fabs(vn[2] * Fn[2])) *
-                              ph.inv_c2);
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-      F[i] = Fn[i];
-      m[i] = mn[i];
-      v[i] = vn[i];
-    }
-    g = gn;
-    w = wn;
-    Ekin = 0.5 * (m[0] * v[0] + m[1] * v[1] + m[2] * v[2]);
-    // |dQ| <= rtol max(|Q_old|, |R|, Q_scale): the three tests of the outer stop
-    double dQ = fabs(Q_new - Q_old);
-    double big = max_nn(max_nn(fabs(Q_old), fabs(R)), Q_scale);
-    if (le_nn(dQ, ph.outer_rtol * big)) {
-      y[0] = Eg;
-      y[1] = m[0]; y[2] = m[1]; y[3] = m[2];
-      y[4] = E;
-      y[5] = F[0]; y[6] = F[1]; y[7] = F[2];
-      if (!pos_finite(E) || !finite_bits(F[0]) || !finite_bits(F[1]) || !finite_bits(F[2]))
-        return RHD_ERR_NONPHYSICAL;
-      return RHD_OK;
-    }
+    if (code == RHD_OK || !warm) return code;
+    warm = settle = false;
   }
-  return RHD_ERR_OUTER;
 }
 
 // Closure tensor D = P/E = dA I + dB Ft Ft^T of a state (E, Ft = F/c).
