@@ -26,6 +26,7 @@ struct ProblemDesc {
   Physics ph;
   double dt;
   long long offset;
+  double wE[2][3], wF[2][3];  // flux_weights of stages 1 and 2
 };
 
 struct WorkItem {
@@ -97,6 +98,11 @@ __global__ void __launch_bounds__(kBatchThreads, 2) batch_kernel(const BatchArgs
     A.eps[1] = B.eps1 ? B.eps1 + off : nullptr;
     A.eps[2] = nullptr;
     A.cost = B.cost ? B.cost + off : nullptr;
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      A.wE[d] = P.wE[STAGE - 1][d];
+      A.wF[d] = P.wF[STAGE - 1][d];
+    }
 #pragma unroll
     for (int q = 0; q < 4; ++q) A.rate[q] = nullptr;
     if (w.kind == 0)
@@ -176,6 +182,8 @@ void fill_desc(const rhd_params* p, ProblemDesc& d) {
   memset(&d, 0, sizeof(d));
   rhd::fill_geometry(p, d.g, d.ph);
   d.dt = rhd_default_dt(p);
+  for (int s = 0; s < 2; ++s)
+    rhd::flux_weights(d.g, d.ph, p->precision == RHD_PREC_MIXED, s == 0 ? d.dt : 0.5 * d.dt, d.wE[s], d.wF[s]);
 }
 
 }  // namespace

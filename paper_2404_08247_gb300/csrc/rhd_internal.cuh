@@ -100,6 +100,11 @@ struct StageArgs {
   double* yo[NY];        // stage output
   const double* eps[3];  // TAU mode: per-face optical-depth factors, or null
                          // (then computed from kappa and rho on the fly)
+  // weights of the face flux differences in the update of E and of the
+  // physical F: u theta dt/dx_d, and c times that, with u the unit of the flux
+  // (chat/2 in FP64, 1 mixed) and theta dt = 1 for rates (stage 0), dt in stage
+  // 1, dt/2 in stage 2 (flux_weights)
+  double wE[3], wF[3];
   double* rate[4];       // transport-only launch: dE/dt, dFx/dt, dFy/dt, dFz/dt
   long long cell_base;   // added to cell indices in failure reports (batched pools)
   DevStatus* st;
@@ -120,6 +125,14 @@ struct StageArgs {
 
 // ghost planes a HALO face holds (the widest face stencil: PPM's 3)
 constexpr int HALO_PLANES = 3;
+
+inline void flux_weights(const Geometry& g, const Physics& ph, bool mixed, double tdt,
+                         double wE[3], double wF[3]) {
+  for (int d = 0; d < 3; ++d) {
+    wE[d] = (mixed ? 1.0 : 0.5 * ph.chat) * g.inv_dx[d] * tdt;
+    wF[d] = ph.c * wE[d];
+  }
+}
 
 // slot pointers of a slot-major buffer of NY * n doubles
 template <typename P>
@@ -181,6 +194,25 @@ __device__ __forceinline__ double dot3(const double a[3], const double b[3]) {
   return fma(a[2], b[2], fma(a[1], b[1], mul(a[0], b[0])));
 }
 
+// x/2, and the magnitude bits of x/4, exactly: the exponent field lowered on
+// the integer pipe (outside the normal range: the product)
+__device__ __forceinline__ double half_of(double x) {
+  const int e = (int)((dbits(x) >> 52) & 0x7ff);
+  return e > 1 && e < 0x7ff ? __longlong_as_double(dbits(x) - (1ll << 52)) : 0.5 * x;
+}
+__device__ __forceinline__ long long quarter_bits(double x) {
+  const long long a = abs_bits(x);
+  return a >= (3ll << 52) && a < kInfBits ? a - (2ll << 52) : abs_bits(0.25 * x);
+}
+// a float as a double, exactly, by integer operations (the conversion where it
+// is zero, subnormal or not finite)
+__device__ __forceinline__ double widen(float f) {
+  const unsigned u = __float_as_uint(f), e = (u >> 23) & 0xffu;
+  if (e == 0u || e == 0xffu) return (double)f;
+  const long long m = ((long long)(u & 0x7fffffffu) << 29) + (896ll << 52);
+  return __longlong_as_double(m | ((long long)(u & 0x80000000u) << 32));
+}
+
 // 1/x to about 2^-21 for x > 0, off the FP64 pipe (outside the single-precision
 // exponent range: the division)
 __device__ __forceinline__ double rcp_approx(double x) {
@@ -225,16 +257,15 @@ __device__ __forceinline__ R half_slope(R um, R u0, R up) {
   return (dm > R(0) && dp > R(0)) ? m : ((dm < R(0) && dp < R(0)) ? -m : R(0));
 }
 
-// double: the same value with the sign tests and the minimum on the integer
-// pipe (0.25 |d- + d+| = |0.25 (d- + d+)| exactly)
+// double: the same value with the sign tests, the quarter and the minimum on
+// the integer pipe
 template <>
 __device__ __forceinline__ double half_slope<double>(double um, double u0, double up) {
   double dm = u0 - um;
   double dp = up - u0;
-  double q = 0.25 * (dm + dp);
   long long bm = dbits(dm), bp = dbits(dp);
   long long am = bm & kMag, ap = bp & kMag;
-  long long m = min(min(am, ap), abs_bits(q));
+  long long m = min(min(am, ap), quarter_bits(dm + dp));
   bool take = ((bm ^ bp) >= 0) & (am != 0) & (ap != 0);  // same sign, both nonzero
   return __longlong_as_double(take ? (m | (bm & ~kMag)) : 0ll);
 }
@@ -383,24 +414,8 @@ __device__ __forceinline__ void ppm_cs_face(const R u[6], R& L, R& Rr) {
 // which needs one square root and one reciprocal and no division by |Ft|
 // (zero flux gives E/3 I without a special case).  Above the free-streaming
 // limit f is clipped to 1: P = E n n = (E/|Ft|^2) Ft Ft^T.  m1_coeffs returns
-// (ha, hb) with P = ha I + hb Ft Ft^T; m1_row returns row d of P.
-template <typename R>
-__device__ __forceinline__ void m1_coeffs(R E, const R Ft[3], R& ha, R& hb) {
-  R F2 = Ft[0] * Ft[0] + Ft[1] * Ft[1] + Ft[2] * Ft[2];
-  R E2 = E * E;
-  if (F2 > E2) {
-    ha = R(0);
-    hb = E / F2;
-  } else {
-    R s = sqrt(R(4) * E2 - R(3) * F2);
-    ha = (s - E) * (R(1) / R(3));
-    hb = R(3) / (R(2) * E + s);
-  }
-}
-
-template <>
-__device__ __forceinline__ void m1_coeffs<double>(double E, const double Ft[3], double& ha,
-                                                  double& hb) {
+// (ha, hb) with P = ha I + hb Ft Ft^T.
+__device__ __forceinline__ void m1_coeffs(double E, const double Ft[3], double& ha, double& hb) {
   const double F2 = dot3(Ft, Ft);
   const double E2 = mul(E, E);
   if (lt_nn(E2, F2)) {
@@ -413,81 +428,60 @@ __device__ __forceinline__ void m1_coeffs<double>(double E, const double Ft[3], 
   }
 }
 
-template <typename R>
-__device__ __forceinline__ void m1_row(int d, R E, const R Ft[3], int closure, R P[3]) {
-  if (closure == RHD_CLOSURE_EDDINGTON) {
-    P[0] = P[1] = P[2] = R(0);
-    P[d] = E * (R(1) / R(3));
-    return;
-  }
-  R ha, hb;
-  m1_coeffs(E, Ft, ha, hb);
-  R t = hb * Ft[d];
-#pragma unroll
-  for (int j = 0; j < 3; ++j) P[j] = t * Ft[j];
-  P[d] += ha;
-}
-
 // ------------------------------------------------------------------- HLL
 // Flux through one face along axis d (Sec. 3.3 Godunov step, Sec. 4.3 wave
 // speeds) for the RSLA system dE/dt = -chat div(Ft), dFt/dt = -chat div(P),
-// from the reconstructed face states L and R (E, Ft).  Reconstructed fluxes
-// above the free-streaming limit are scaled back onto |Ft| = E.  Symmetric
-// speeds S_R = -S_L = chat sqrt(max(D_dd,L, D_dd,R, 1/3)), D = P/E, so HLL is
+// from the reconstructed face states L and R (E, Ft), in units of chat/2 (the
+// update's weights hold the factor).  Reconstructed fluxes above the
+// free-streaming limit are scaled back onto |Ft| = E.  Symmetric speeds S_R =
+// -S_L = chat sqrt(max(D_dd,L, D_dd,R, 1/3)), D = P/E, so HLL is
 //   Phi = (Phi_L + Phi_R)/2 - S (U_R - U_L)/2,
 // with the optical-depth factor eps on the energy part (1 for HLL NONE).
 // Returns false for a face state with E <= 0 (or NaN).
-// a > 0 and a < b for a, b >= 0 in the transport precision (integer pipe for
-// double, plain compares for float)
-template <typename R>
-__device__ __forceinline__ bool positive(R a) {
-  if constexpr (sizeof(R) == 8) return dbits(a) > 0 && dbits(a) < kInfBits;
-  else return a > R(0);
-}
-template <typename R>
-__device__ __forceinline__ bool less_nn(R a, R b) {
-  if constexpr (sizeof(R) == 8) return lt_nn(a, b);
-  else return a < b;
+
+// One side: the free-streaming limit applied to q = (E, Ft), and row d of its
+// P.  With h = s/2 = sqrt(E^2 - 3/4 |Ft|^2) the closure of m1_coeffs is P =
+// (2h - E)/3 I + 3/2/(E + h) Ft Ft^T; E^2 and |Ft|^2 serve the limit as well
+// (a flux scaled back has |Ft| = E, so P = E n n).
+__device__ __forceinline__ void face_side(int d, double q[4], int closure, double P[3]) {
+  const double E = q[0], E2 = mul(E, E);
+  double F2 = dot3(q + 1, q + 1);
+  if (lt_nn(E2, F2)) {
+    const double sc = mul(E, rsqrt_pos(F2));
+#pragma unroll
+    for (int j = 0; j < 3; ++j) q[1 + j] = mul(q[1 + j], sc);
+    F2 = E2;
+  }
+  if (closure == RHD_CLOSURE_EDDINGTON) {
+    P[0] = P[1] = P[2] = 0.0;
+    P[d] = mul(E, 1.0 / 3.0);
+    return;
+  }
+  const double h = sqrt_pos(fma(-0.75, F2, E2));
+  const double ha = mul(fma(2.0, h, -E), 1.0 / 3.0);
+  const double t = mul(mul(1.5, rcp_pos(add(E, h))), q[1 + d]);
+#pragma unroll
+  for (int j = 0; j < 3; ++j) P[j] = j == d ? fma(t, q[1 + j], ha) : mul(t, q[1 + j]);
 }
 
-template <typename R>
-__device__ __forceinline__ bool hll_states(int d, R L[4], R Rr[4], R eps, R chat,
-                                           int closure, R out[4]) {
-  if (!positive(L[0]) || !positive(Rr[0])) {
-    out[0] = out[1] = out[2] = out[3] = R(0);
+__device__ __forceinline__ bool hll_states(int d, double L[4], double R[4], double eps,
+                                           int closure, double out[4]) {
+  if (!pos_finite(L[0]) || !pos_finite(R[0])) {
+    out[0] = out[1] = out[2] = out[3] = 0.0;
     return false;
   }
-  {
-    R n2 = L[1] * L[1] + L[2] * L[2] + L[3] * L[3];
-    if (less_nn(L[0] * L[0], n2)) {
-      R sc;
-      if constexpr (sizeof(R) == 8) sc = L[0] * rsqrt_pos(n2);
-      else sc = L[0] / sqrt(n2);
-      L[1] *= sc; L[2] *= sc; L[3] *= sc;
-    }
-    n2 = Rr[1] * Rr[1] + Rr[2] * Rr[2] + Rr[3] * Rr[3];
-    if (less_nn(Rr[0] * Rr[0], n2)) {
-      R sc;
-      if constexpr (sizeof(R) == 8) sc = Rr[0] * rsqrt_pos(n2);
-      else sc = Rr[0] / sqrt(n2);
-      Rr[1] *= sc; Rr[2] *= sc; Rr[3] *= sc;
-    }
-  }
-  R PL[3], PR[3];
-  m1_row(d, L[0], &L[1], closure, PL);
-  m1_row(d, Rr[0], &Rr[1], closure, PR);
-  // largest of D_dd,L, D_dd,R and 1/3 without dividing each (P_dd >= 0)
-  R num = PL[d], den = L[0];
-  if (less_nn(PL[d] * Rr[0], PR[d] * L[0])) { num = PR[d]; den = Rr[0]; }
-  if (less_nn(R(3) * num, den)) { num = R(1); den = R(3); }
-  R S;
-  if constexpr (sizeof(R) == 8) S = chat * num * rsqrt_pos(num * den);  // sqrt(num/den)
-  else S = chat * sqrt(num / den);
-  R hc = R(0.5) * chat;
-  R hS = R(0.5) * S;
-  out[0] = hc * (L[1 + d] + Rr[1 + d]) - eps * hS * (Rr[0] - L[0]);
+  double PL[3], PR[3];
+  face_side(d, L, closure, PL);
+  face_side(d, R, closure, PR);
+  // S/chat from the largest of D_dd,L, D_dd,R and 1/3, without dividing each
+  // (P_dd >= 0): sqrt(num/den) = num/sqrt(num den)
+  double num = PL[d], den = L[0];
+  if (lt_nn(mul(PL[d], R[0]), mul(PR[d], L[0]))) { num = PR[d]; den = R[0]; }
+  if (lt_nn(mul(3.0, num), den)) { num = 1.0; den = 3.0; }
+  const double S = mul(num, rsqrt_pos(mul(num, den)));
+  out[0] = fma(-mul(eps, S), sub(R[0], L[0]), add(L[1 + d], R[1 + d]));
 #pragma unroll
-  for (int j = 0; j < 3; ++j) out[1 + j] = hc * (PL[j] + PR[j]) - hS * (Rr[1 + j] - L[1 + j]);
+  for (int j = 0; j < 3; ++j) out[1 + j] = fma(-S, sub(R[1 + j], L[1 + j]), add(PL[j], PR[j]));
   return true;
 }
 
@@ -521,16 +515,16 @@ __device__ __forceinline__ void m1_dev_row(int d, float E, const float Ft[3], in
 
 // HLL flux of hll_states in mixed precision.  The isotropic part of the
 // normal momentum flux, hc (E_L + E_R)/3 (hc = chat/2), is linear in the face
-// states: it is returned in double (iso, from the exact single-precision face
-// energies and chat6 = chat/6 in double) and left out of out[1 + d], which
+// states: iso = E_L + E_R is returned in double (the exact single-precision
+// face energies, widened off the FP64 pipe) and left out of out[1 + d], which
 // carries the single-precision rest.  The flux of F along d is out[1 + d] +
-// iso.  Rounding P_dd in single precision at every face gives each face an
+// chat/6 iso (units of 1, where the double-precision flux has chat/2).  Rounding P_dd in single precision at every face gives each face an
 // independent error of an ulp of E/3, which the flux difference turns into
 // an error of the flux update of order 1e-7 E/|Ft| relative; near isotropy
 // (|Ft| << E) that is the dominant single-precision error.
 __device__ __forceinline__ bool hll_states_mixed(int d, float L[4], float Rr[4], float eps,
-                                                 float chat, int closure, double chat6,
-                                                 float out[4], double& iso) {
+                                                 float chat, int closure, float out[4],
+                                                 double& iso) {
   iso = 0.0;
   if (!(L[0] > 0.f) || !(Rr[0] > 0.f)) {
     out[0] = out[1] = out[2] = out[3] = 0.f;
@@ -560,20 +554,20 @@ __device__ __forceinline__ bool hll_states_mixed(int d, float L[4], float Rr[4],
   out[0] = hc * (L[1 + d] + Rr[1 + d]) - eps * hS * (Rr[0] - L[0]);
 #pragma unroll
   for (int j = 0; j < 3; ++j) out[1 + j] = hc * (DL[j] + DR[j]) - hS * (Rr[1 + j] - L[1 + j]);
-  iso = chat6 * ((double)L[0] + (double)Rr[0]);
+  iso = widen(L[0]) + widen(Rr[0]);
   return true;
 }
 
-// The face flux in the transport precision R: hll_states for double (iso =
-// 0, unused), hll_states_mixed for float.
+// The face flux in the transport precision R: hll_states for double (units of
+// chat/2; iso = 0, unused), hll_states_mixed for float.
 template <typename R>
 __device__ __forceinline__ bool face_hll(int d, R L[4], R Rr[4], R eps, R chat, int closure,
-                                         double chat6, R out[4], double& iso) {
+                                         R out[4], double& iso) {
   if constexpr (sizeof(R) == 8) {
     iso = 0.0;
-    return hll_states<R>(d, L, Rr, eps, chat, closure, out);
+    return hll_states(d, L, Rr, eps, closure, out);
   } else {
-    return hll_states_mixed(d, L, Rr, eps, chat, closure, chat6, out, iso);
+    return hll_states_mixed(d, L, Rr, eps, chat, closure, out, iso);
   }
 }
 

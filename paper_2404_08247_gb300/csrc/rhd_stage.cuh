@@ -48,6 +48,8 @@ static cudaError_t launch_nd(const StageArgs& A, cudaStream_t s, int b0, int b1)
   nb[NDIM - 1] = (unsigned)(b1 - b0);
   StageArgs a = A;
   a.blk_off = b0;
+  flux_weights(A.g, A.ph, sizeof(R) == sizeof(float),
+               STAGE == 0 ? 1.0 : STAGE == 1 ? A.dt : 0.5 * A.dt, a.wE, a.wF);
   stage_kernel<STAGE, NDIM, R, GEN, PPM><<<dim3(nb[0], nb[1], nb[2]), T::TX * T::TY, S::BYTES,
                                            s>>>(a);
   return cudaGetLastError();

@@ -102,7 +102,15 @@ struct SmemT {
       SORT_ALIAS ? sizeof(R) * RING : ISO_OFF + sizeof(double) * (FXI + FYI);
   static constexpr size_t SORT_I_OFF = ISO_OFF + sizeof(double) * (FXI + FYI) +
                                        (SORT_ALIAS ? 0 : sizeof(double) * 8 * T::NT);
-  static constexpr size_t BYTES = SORT_I_OFF + sizeof(int) * (3 * T::NT + (T::NT / 32) * NB);
+  static constexpr size_t SORT_END = SORT_I_OFF + sizeof(int) * (3 * T::NT + (T::NT / 32) * NB);
+  // FP64 PLM: half slopes along x of the tile's cells and one beyond on each
+  // side, and along y, so that each is computed once and not for both faces
+  // of its cell
+  static constexpr bool SLOPES = !T::PPM && sizeof(R) == sizeof(double);
+  static constexpr int SX = SLOPES ? T::TY * (T::TX + 2) : 0;            // per field
+  static constexpr int SY = SLOPES && T::NDIM >= 2 ? (T::TY + 2) * T::TX : 0;
+  static constexpr size_t SLOPE_OFF = (SORT_END + 15) / 16 * 16;
+  static constexpr size_t BYTES = SLOPE_OFF + sizeof(double) * 4 * (SX + SY);
 };
 
 // Coordinate x >= -3 folded onto [0, n) by the boundary condition (padding
@@ -186,8 +194,8 @@ __device__ __forceinline__ double face_eps(const StageArgs& A, int d, int cx, in
 }
 
 // Mixed precision: x as a pair of floats with hi + lo = x to 2^-47 |x|.  hi
-// is x with its mantissa cut to 24 bits (integer operations; exact in float
-// within the float exponent range), lo = x - hi rounded to float.  A
+// is x with its mantissa cut to 24 bits, lo the rest rounded to float, both by
+// integer operations within the float exponent range.  A
 // difference of two neighbours, (b_hi - a_hi) + (b_lo - a_lo), is then good
 // to single precision of the difference itself, where the difference of the
 // rounded values would carry an error of an ulp of the values: the MC slopes
@@ -195,11 +203,12 @@ __device__ __forceinline__ double face_eps(const StageArgs& A, int d, int cx, in
 __device__ __forceinline__ void split_hilo(double x, float& hi, float& lo) {
   const long long b = __double_as_longlong(x);
   const int e = (int)((b >> 52) & 0x7ff);
-  if (e >= 1023 - 126 && e <= 1023 + 127) {
-    const double xt = __longlong_as_double(b & ~((1ll << 29) - 1));
-    hi = __uint_as_float((unsigned)((b >> 32) & 0x80000000ll) |
-                         ((unsigned)(e - 1023 + 127) << 23) | (unsigned)((b >> 29) & 0x7fffff));
-    lo = (float)(x - xt);
+  if (e >= 1023 - 70 && e <= 1023 + 126) {
+    const unsigned sign = (unsigned)((b >> 32) & 0x80000000ll);
+    hi = __uint_as_float(sign | ((unsigned)(e - 896) << 23) | (unsigned)((b >> 29) & 0x7fffff));
+    // the low 29 bits, in units of 2^(e - 1023 - 52)
+    lo = (float)(unsigned)(b & 0x1fffffffll) *
+         __uint_as_float(sign | ((unsigned)(e - 896 - 52) << 23));
   } else {
     hi = (float)x;
     lo = (float)(x - (double)hi);
@@ -344,10 +353,11 @@ __device__ __forceinline__ void ppm_states(const R u[6][4], R L[4], R Rr[4], boo
 
 // flux through the face between plane cells c - st and c (stride st); cs:
 // PPM tiles with the Colella-Sekora limiter; iso: see face_hll
+// (sl, sr: the half slopes of cells c - st and c, field q at q * sn; FP64 PLM)
 template <class T, typename R>
 __device__ __forceinline__ bool plane_face(const R* pl, int c, int st, int d, R eps, R chat,
-                                           int closure, double chat6, R out[4], double& iso,
-                                           bool cs = false) {
+                                           int closure, R out[4], double& iso, const double* sl,
+                                           const double* sr, int sn, bool cs = false) {
   R L[4], Rr[4];
   if constexpr (T::PPM) {
     R u[6][4];
@@ -370,18 +380,16 @@ __device__ __forceinline__ bool plane_face(const R* pl, int c, int st, int d, R 
       Rr[q] = hb[q] + (lb[q] - half_slope_d(d1, d2));
     }
   } else {
-    R am[4], a[4], b[4], bp[4];
-    cell_of<T, R>(pl, c - 2 * st, am);
+    R a[4], b[4];
     cell_of<T, R>(pl, c - st, a);
     cell_of<T, R>(pl, c, b);
-    cell_of<T, R>(pl, c + st, bp);
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-      L[q] = a[q] + half_slope(am[q], a[q], b[q]);
-      Rr[q] = b[q] - half_slope(a[q], b[q], bp[q]);
+      L[q] = a[q] + sl[q * sn];
+      Rr[q] = b[q] - sr[q * sn];
     }
   }
-  return face_hll<R>(d, L, Rr, eps, chat, closure, chat6, out, iso);
+  return face_hll<R>(d, L, Rr, eps, chat, closure, out, iso);
 }
 
 // One cell (E, F/c) of the own column (cx, cy inside the grid) at plane zg,
@@ -615,7 +623,9 @@ __device__ __forceinline__ void stage_tile(const StageArgs& A, int x0, int y0, i
     }
   }
   const R chat = (R)ph.chat;
-  const double chat6 = ph.chat * (1.0 / 6.0);
+  const double chat6 = ph.chat * (1.0 / 6.0);  // weight of the mixed iso parts
+  double* sx = reinterpret_cast<double*>(smem_raw + S::SLOPE_OFF);  // FP64 PLM only
+  double* sy = sx + 4 * S::SX;
   const int tx = threadIdx.x % TX, ty = threadIdx.x / TX;
   const int ix = x0 + tx, iy = y0 + ty;
   const bool col = ix < g.n[0] && (NDIM < 2 || iy < g.n[1]);
@@ -677,7 +687,7 @@ __device__ __forceinline__ void stage_tile(const StageArgs& A, int x0, int y0, i
       }
     }
     R eps = (R)face_eps(A, 2, cx, cy, kbeg - 1);
-    zbad = !face_hll<R>(2, L, Rr, eps, chat, ph.closure, chat6, zlo, zlo_iso);
+    zbad = !face_hll<R>(2, L, Rr, eps, chat, ph.closure, zlo, zlo_iso);
     for (int o = 0; o <= 2; ++o)
       load_plane<T, R, GEN>(A, ring, ring_slot<T>(kbeg + o), kbeg + o, x0, y0);
   } else if constexpr (NDIM == 3) {
@@ -714,7 +724,7 @@ __device__ __forceinline__ void stage_tile(const StageArgs& A, int x0, int y0, i
       }
     }
     R eps = (R)face_eps(A, 2, cx, cy, kbeg - 1);
-    zbad = !face_hll<R>(2, L, Rr, eps, chat, ph.closure, chat6, zlo, zlo_iso);
+    zbad = !face_hll<R>(2, L, Rr, eps, chat, ph.closure, zlo, zlo_iso);
     __syncthreads();  // plane kbeg-2's slot is reloaded by the first iteration
   }
 
@@ -768,7 +778,7 @@ __device__ __forceinline__ void stage_tile(const StageArgs& A, int x0, int y0, i
         }
       }
       R eps = (R)face_eps(A, 2, cx, cy, k);
-      zbad = !face_hll<R>(2, L, Rr, eps, chat, ph.closure, chat6, zhi, zhi_iso);
+      zbad = !face_hll<R>(2, L, Rr, eps, chat, ph.closure, zhi, zhi_iso);
       bad = bad || zbad;
     } else if constexpr (NDIM == 3) {
       R L[4], Rr[4];
@@ -797,8 +807,34 @@ __device__ __forceinline__ void stage_tile(const StageArgs& A, int x0, int y0, i
         }
       }
       R eps = (R)face_eps(A, 2, cx, cy, k);
-      zbad = !face_hll<R>(2, L, Rr, eps, chat, ph.closure, chat6, zhi, zhi_iso);
+      zbad = !face_hll<R>(2, L, Rr, eps, chat, ph.closure, zhi, zhi_iso);
       bad = bad || zbad;
+    }
+
+    // ---- FP64 PLM: half slopes of plane k, each thread its own cell's, then
+    // those of the cells next to the tile
+    if constexpr (S::SLOPES) {
+      auto slope = [&](int c, int st, double* out, int sn) {
+        double um[4], u0[4], up[4];
+        cell_of<T, R>(pl, c - st, um);
+        cell_of<T, R>(pl, c, u0);
+        cell_of<T, R>(pl, c + st, up);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) out[q * sn] = half_slope(um[q], u0[q], up[q]);
+      };
+      slope(own, 1, sx + ty * (TX + 2) + tx + 1, S::SX);
+      if (NDIM >= 2) slope(own, S::PW, sy + (ty + 1) * TX + tx, S::SY);
+      constexpr int NY2 = NDIM >= 2 ? 2 * TX : 0;
+      for (int i = threadIdx.x; i < NY2 + 2 * TY; i += NT) {
+        if (NDIM >= 2 && i < NY2) {  // rows -1 and TY
+          const int r = i < TX ? -1 : TY, x = i < TX ? i : i - TX;
+          slope(x + T::HX + (r + T::HY) * S::PW, S::PW, sy + (r + 1) * TX + x, S::SY);
+        } else {  // columns -1 and TX
+          const int j = i - NY2, r = j >> 1, x = (j & 1) ? TX : -1;
+          slope(x + T::HX + (r + T::HY) * S::PW, 1, sx + r * (TX + 2) + x + 1, S::SX);
+        }
+      }
+      __syncthreads();
     }
 
     // ---- x-faces of plane k: face f lies between tile cells fi-1 and fi
@@ -811,7 +847,9 @@ __device__ __forceinline__ void stage_tile(const StageArgs& A, int x0, int y0, i
       R eps = real ? (R)face_eps(A, 0, xl, yr, k) : R(1);
       R out[4];
       double iso;
-      if (!plane_face<T, R>(pl, c, 1, 0, eps, chat, ph.closure, chat6, out, iso, cs) && real) {
+      const double* sl = sx + fj * (TX + 2) + fi;
+      if (!plane_face<T, R>(pl, c, 1, 0, eps, chat, ph.closure, out, iso, sl, sl + 1, S::SX, cs) &&
+          real) {
         // a face with E <= 0 poisons both neighbours' fluxes
 #pragma unroll
         for (int q = 0; q < 4; ++q) out[q] = (R)__longlong_as_double(0x7ff8000000000000ll);
@@ -830,7 +868,9 @@ __device__ __forceinline__ void stage_tile(const StageArgs& A, int x0, int y0, i
         R eps = real ? (R)face_eps(A, 1, xr, yl, k) : R(1);
         R out[4];
         double iso;
-        if (!plane_face<T, R>(pl, c, S::PW, 1, eps, chat, ph.closure, chat6, out, iso, cs) &&
+        const double* sl = sy + fj * TX + fi;
+        if (!plane_face<T, R>(pl, c, S::PW, 1, eps, chat, ph.closure, out, iso, sl, sl + TX, S::SY,
+                              cs) &&
             real) {
 #pragma unroll
           for (int q = 0; q < 4; ++q) out[q] = (R)__longlong_as_double(0x7ff8000000000000ll);
@@ -854,61 +894,54 @@ __device__ __forceinline__ void stage_tile(const StageArgs& A, int x0, int y0, i
     const bool rk2 = GEN && ph.scheme == RHD_SCHEME_RK2_SSP;
     if (col) {
       idx = ix + g.n[0] * (iy + g.n[1] * k);
-      double rate[4];
-      const int fl = tx + ty * (TX + 1);
+      // the explicit state y* (stage 1), y** (stage 2), or 0 for the rates
+      if (STAGE == 1) {
+#pragma unroll
+        for (int q = 0; q < 8; ++q) y[q] = RHD_LD(A.st, A.yt[q], idx, g.ncell);
+      } else if (STAGE == 2) {
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+          y[q] = half_of(add(RHD_LD(A.st, A.yn[q], idx, g.ncell),
+                             RHD_LD(A.st, A.yt[q], idx, g.ncell)));
+      }
       // flux differences in double: the difference of two floats is exact in
       // double, so the update telescopes across cells in both precisions
+      const int fl = tx + ty * (TX + 1), fb = tx + ty * TX;
+      auto diff = [](R hi, R lo) {
+        if constexpr (MIXED) return sub(widen(hi), widen(lo));
+        else return sub(hi, lo);
+      };
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
+        double& yq = y[Y_ERAD + q];
+        const double* w = q == 0 ? A.wE : A.wF;
         const R* fq = fxs + q * TY * (TX + 1);
-        double df = (double)fq[fl + 1] - (double)fq[fl];
-        if (MIXED && q == 1) df += fxi[fl + 1] - fxi[fl];
-        rate[q] = -df * g.inv_dx[0];
-      }
-      if (NDIM >= 2) {
-        const int fb = tx + ty * TX;
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const R* fq = fys + q * (TY + 1) * TX;
-          double df = (double)fq[fb + TX] - (double)fq[fb];
-          if (MIXED && q == 2) df += fyi[fb + TX] - fyi[fb];
-          rate[q] -= df * g.inv_dx[1];
+        double df = diff(fq[fl + 1], fq[fl]);
+        if (MIXED && q == 1) df = fma(sub(fxi[fl + 1], fxi[fl]), chat6, df);
+        yq = fma(-df, w[0], yq);
+        if (NDIM >= 2) {
+          const R* gq = fys + q * (TY + 1) * TX;
+          df = diff(gq[fb + TX], gq[fb]);
+          if (MIXED && q == 2) df = fma(sub(fyi[fb + TX], fyi[fb]), chat6, df);
+          yq = fma(-df, w[1], yq);
         }
-      }
-      if (NDIM == 3) {
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          double df = (double)zhi[q] - (double)zlo[q];
-          if (MIXED && q == 3) df += zhi_iso - zlo_iso;
-          rate[q] -= df * g.inv_dx[2];
+        if (NDIM == 3) {
+          df = diff(zhi[q], zlo[q]);
+          if (MIXED && q == 3) df = fma(sub(zhi_iso, zlo_iso), chat6, df);
+          yq = fma(-df, w[2], yq);
         }
+        bad = bad || !finite_bits(yq);
       }
-      bad = bad || !isfinite(rate[0]) || !isfinite(rate[1]) || !isfinite(rate[2]) ||
-            !isfinite(rate[3]);
 
       if (STAGE == 0) {
         // transport only: s(y) of eq. (yrsla) for E and the physical flux F
-        RHD_ST(A.st, A.rate[0], idx, g.ncell, rate[0]);
 #pragma unroll
-        for (int j = 0; j < 3; ++j) RHD_ST(A.st, A.rate[1 + j], idx, g.ncell, ph.c * rate[1 + j]);
+        for (int q = 0; q < 4; ++q) RHD_ST(A.st, A.rate[q], idx, g.ncell, y[Y_ERAD + q]);
         if (bad) {
           atomicMin(&A.st->fail_key, ((unsigned long long)(A.cell_base + idx) << 8) | RHD_ERR_NONPHYSICAL);
           A.st->fail_step = A.step;
           A.st->fail_stage = 0;
         }
-      } else if (STAGE == 1) {
-#pragma unroll
-        for (int q = 0; q < 8; ++q) y[q] = RHD_LD(A.st, A.yt[q], idx, g.ncell);
-        y[Y_ERAD] += A.dt * rate[0];
-#pragma unroll
-        for (int j = 0; j < 3; ++j) y[Y_FX + j] += A.dt * ph.c * rate[1 + j];
-      } else {
-#pragma unroll
-        for (int q = 0; q < 8; ++q)
-          y[q] = 0.5 * (RHD_LD(A.st, A.yn[q], idx, g.ncell) + RHD_LD(A.st, A.yt[q], idx, g.ncell));
-        y[Y_ERAD] += 0.5 * A.dt * rate[0];
-#pragma unroll
-        for (int j = 0; j < 3; ++j) y[Y_FX + j] += 0.5 * A.dt * ph.c * rate[1 + j];
       }
       rho = RHD_LD(A.st, A.rho, idx, g.ncell);
       chi = RHD_LD(A.st, A.kappa, idx, g.ncell) * rho;
