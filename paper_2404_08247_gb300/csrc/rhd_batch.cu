@@ -49,7 +49,6 @@ struct BatchArgs {
   const double* eps1;
   DevStatus* st;
   int step;
-  unsigned char* cost;  // this stage's per-cell solve costs (pooled), or null
 };
 
 using Tile1 = TileT<1, 256, 1, 1>;
@@ -66,6 +65,8 @@ template <int STAGE, class T2, typename R, bool GEN, bool PPMX>
 __global__ void __launch_bounds__(kBatchThreads, 2) batch_kernel(const BatchArgs B) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ int s_item, s_skip;
+  __shared__ __align__(16) unsigned char s_args[sizeof(StageArgs)];
+  StageArgs& A = *reinterpret_cast<StageArgs*>(s_args);
   if (threadIdx.x == 0) s_skip = (B.st->fail_key != ~0ull) ? 1 : 0;
   __syncthreads();
   if (s_skip) return;  // a previous launch of this batch failed
@@ -78,42 +79,42 @@ __global__ void __launch_bounds__(kBatchThreads, 2) batch_kernel(const BatchArgs
     if (it >= B.nitems) break;
     const WorkItem w = B.items[it];
     const ProblemDesc& P = B.probs[w.prob];
-    StageArgs A;
-    A.g = P.g;
-    A.ph = P.ph;
-    A.dt = P.dt;
-    A.step = B.step;
-    A.st = B.st;
-    A.cell_base = P.offset;
-    const long long off = P.offset;
-#pragma unroll
-    for (int q = 0; q < NY; ++q) {
-      A.yt[q] = B.yt + q * B.ntot + off;
-      A.yn[q] = B.yn + q * B.ntot + off;
-      A.yo[q] = B.yo + q * B.ntot + off;
+    // the item's arguments in shared memory, where the tile reads them as the
+    // grid kernels read their launch arguments: held in registers they cost
+    // 700 bytes of spills a thread
+    if (threadIdx.x == 0) {
+      A.g = P.g;
+      A.ph = P.ph;
+      A.dt = P.dt;
+      A.step = B.step;
+      A.st = B.st;
+      A.cell_base = P.offset;
+      const long long off = P.offset;
+      for (int q = 0; q < NY; ++q) {
+        A.yt[q] = B.yt + q * B.ntot + off;
+        A.yn[q] = B.yn + q * B.ntot + off;
+        A.yo[q] = B.yo + q * B.ntot + off;
+      }
+      A.rho = B.rho + off;
+      A.kappa = B.kappa + off;
+      A.eps[0] = B.eps0 ? B.eps0 + off : nullptr;
+      A.eps[1] = B.eps1 ? B.eps1 + off : nullptr;
+      A.eps[2] = nullptr;
+      for (int d = 0; d < 3; ++d) {
+        A.wE[d] = P.wE[STAGE - 1][d];
+        A.wF[d] = P.wF[STAGE - 1][d];
+      }
     }
-    A.rho = B.rho + off;
-    A.kappa = B.kappa + off;
-    A.eps[0] = B.eps0 ? B.eps0 + off : nullptr;
-    A.eps[1] = B.eps1 ? B.eps1 + off : nullptr;
-    A.eps[2] = nullptr;
-    A.cost = B.cost ? B.cost + off : nullptr;
-#pragma unroll
-    for (int d = 0; d < 3; ++d) {
-      A.wE[d] = P.wE[STAGE - 1][d];
-      A.wF[d] = P.wF[STAGE - 1][d];
-    }
-#pragma unroll
-    for (int q = 0; q < 4; ++q) A.rate[q] = nullptr;
+    __syncthreads();
     if (w.kind == 0)
-      stage_tile<STAGE, Tile1, R, GEN>(A, w.x0, 0, 0, smem_raw, ts);
+      stage_tile<STAGE, Tile1, R, GEN, true>(A, w.x0, 0, 0, smem_raw, ts);
     else if (!PPMX || w.kind == 1)
-      stage_tile<STAGE, T2, R, GEN>(A, w.x0, w.y0, 0, smem_raw, ts);
+      stage_tile<STAGE, T2, R, GEN, true>(A, w.x0, w.y0, 0, smem_raw, ts);
     else if constexpr (PPMX) {
       if (w.kind == 2)
-        stage_tile<STAGE, Tile1P, R, true>(A, w.x0, 0, 0, smem_raw, ts);
+        stage_tile<STAGE, Tile1P, R, true, true>(A, w.x0, 0, 0, smem_raw, ts);
       else
-        stage_tile<STAGE, Tile2P, R, true>(A, w.x0, w.y0, 0, smem_raw, ts);
+        stage_tile<STAGE, Tile2P, R, true, true>(A, w.x0, w.y0, 0, smem_raw, ts);
     }
   }
   flush_stats<kBatchThreads>(B.st, ts);
@@ -201,7 +202,6 @@ struct rhd_batch {
   double* rho = nullptr;
   double* kappa = nullptr;
   double* eps[2] = {nullptr, nullptr};
-  unsigned char* cost = nullptr;  // solve costs of stage 1 and 2 (2 ntot bytes)
   ProblemDesc* d_desc = nullptr;
   WorkItem* d_items = nullptr;
   int nitems = 0;
@@ -263,7 +263,6 @@ static void batch_release(rhd_batch* b) {
   cudaFree(b->yhalf);
   cudaFree(b->rho);
   cudaFree(b->kappa);
-  cudaFree(b->cost);
   cudaFree(b->eps[0]);
   cudaFree(b->eps[1]);
   cudaFree(b->d_desc);
@@ -351,8 +350,6 @@ rhd_status rhd_batch_init(const rhd_params* probs, int nprob, rhd_batch** out) {
   if (e == cudaSuccess) e = cudaMalloc(&b->yhalf, sizeof(double) * NY * N);
   if (e == cudaSuccess) e = cudaMalloc(&b->rho, sizeof(double) * N);
   if (e == cudaSuccess) e = cudaMalloc(&b->kappa, sizeof(double) * N);
-  if (e == cudaSuccess) e = cudaMalloc(&b->cost, 2 * N);
-  if (e == cudaSuccess) e = cudaMemset(b->cost, 0, 2 * N);
   if (any_tau) {
     if (e == cudaSuccess) e = cudaMalloc(&b->eps[0], sizeof(double) * N);
     if (e == cudaSuccess) e = cudaMalloc(&b->eps[1], sizeof(double) * N);
@@ -504,13 +501,11 @@ static cudaError_t enqueue_steps(rhd_batch* b, int nsteps, int cur0, cudaStream_
     B.yt = b->ybuf[cur];
     B.yn = b->ybuf[cur];
     B.yo = b->yhalf;
-    B.cost = b->cost;
     e = cudaMemsetAsync(b->d_counter, 0, sizeof(int), cs);
     if (e == cudaSuccess)
       e = launch_batch(1, b->precision, b->general, b->ppm, b->tile2d, B, grid, cs);
     B.yt = b->yhalf;
     B.yo = b->ybuf[cur ^ 1];
-    B.cost = b->cost + b->ntot;
     if (e == cudaSuccess) e = cudaMemsetAsync(b->d_counter, 0, sizeof(int), cs);
     if (e == cudaSuccess)
       e = launch_batch(2, b->precision, b->general, b->ppm, b->tile2d, B, grid, cs);

@@ -87,29 +87,13 @@ struct SmemT {
   static constexpr int FXI = ISO ? T::TY * (T::TX + 1) : 0;
   static constexpr int FYI = ISO && T::NDIM >= 2 ? (T::TY + 1) * T::TX : 0;
   static constexpr size_t ISO_OFF = sizeof(R) * (RING + FX + FY + CZ);
-  // local solves in cost order (stages 1 and 2, where the launch supplies
-  // the predicted costs): per slot the explicit state (8 doubles,
-  // slot-minor), then per slot the solve flag and source thread / the
-  // status, the Newton and outer counts, and the per-warp counts of each cost
-  // bucket.  The FP64 3-D PPM tile, whose two blocks per SM leave no room for
-  // more, stages the states in its face-flux arrays, which hold nothing
-  // between a plane's flux differences and the next plane's faces.
-  static constexpr int NB = 32;  // cost buckets
-  static constexpr bool SORT_ALIAS = T::PPM && T::NDIM == 3 && sizeof(R) == sizeof(double);
-  static_assert(!SORT_ALIAS || sizeof(R) * (FX + FY) >= sizeof(double) * 8 * T::NT,
-                "the face-flux arrays hold the staged states");
-  static constexpr size_t SORT_Y_OFF =
-      SORT_ALIAS ? sizeof(R) * RING : ISO_OFF + sizeof(double) * (FXI + FYI);
-  static constexpr size_t SORT_I_OFF = ISO_OFF + sizeof(double) * (FXI + FYI) +
-                                       (SORT_ALIAS ? 0 : sizeof(double) * 8 * T::NT);
-  static constexpr size_t SORT_END = SORT_I_OFF + sizeof(int) * (3 * T::NT + (T::NT / 32) * NB);
   // FP64 PLM: half slopes along x of the tile's cells and one beyond on each
   // side, and along y, so that each is computed once and not for both faces
   // of its cell
   static constexpr bool SLOPES = !T::PPM && sizeof(R) == sizeof(double);
   static constexpr int SX = SLOPES ? T::TY * (T::TX + 2) : 0;            // per field
   static constexpr int SY = SLOPES && T::NDIM >= 2 ? (T::TY + 2) * T::TX : 0;
-  static constexpr size_t SLOPE_OFF = (SORT_END + 15) / 16 * 16;
+  static constexpr size_t SLOPE_OFF = ISO_OFF + sizeof(double) * (FXI + FYI);
   static constexpr size_t BYTES = SLOPE_OFF + sizeof(double) * 4 * (SX + SY);
 };
 
@@ -445,144 +429,6 @@ __device__ __forceinline__ void column_cell(const StageArgs& A, int cx, int cy, 
 }
 
 // Per-thread iteration statistics of the cells a thread has solved.
-// ------------------------------------------------ local solves in cost order
-// Shared arrays of the sorted solves: 8 doubles per slot (the explicit state
-// y*), then per slot the solve flag and source thread (in) / the status
-// (out), the Newton and the outer counts, then the per-warp counts of each
-// cost bucket.
-template <class T, typename R>
-struct SortSmem {
-  double* v;
-  int* flag;
-  int* nn;
-  int* no;
-  int* tab;
-  __device__ __forceinline__ explicit SortSmem(unsigned char* smem) {
-    using S = SmemT<T, R>;
-    v = reinterpret_cast<double*>(smem + S::SORT_Y_OFF);
-    flag = reinterpret_cast<int*>(smem + S::SORT_I_OFF);
-    nn = flag + T::NT;
-    no = nn + T::NT;
-    tab = no + T::NT;
-  }
-};
-
-// Solve cost of a cell as kept between steps: its outer passes (1..8) in the
-// top 3 bits, its Newton updates (0..31) in the low 5; 0 before the first.
-__device__ __forceinline__ unsigned char cost_byte(int nn, int no) {
-  return (unsigned char)((min(max(no, 1), 8) - 1) << 5 | min(nn, 31));
-}
-
-// Cost bucket of a kept cost: nn + 4 no - 8, within [0, 31] (the work of a
-// Newton update counting 1 and of an outer pass about 4).
-__device__ __forceinline__ int cost_key(int b) {
-  if (b == 0) return 0;
-  const int no = (b >> 5) + 1, nn = b & 31;
-  return max(0, min(31, nn + 4 * no - 8));
-}
-
-// Slot of this thread's cell in the block's cost order: a stable counting
-// sort on the cost bucket of the previous step's cost (cells without a solve
-// in bucket 0).  Sorted rank r goes to warp r / 32 in the first half of
-// the warps and to the mirrored warp in the second (ranks 128..255 of 256 to
-// warps 7..4), so that each of the SM's schedulers (warp w runs on scheduler
-// w mod 4) holds one cheaper and one dearer warp of the block.  The bucket
-// counts must be zero on entry; every thread of the block calls this.
-template <class T, typename R>
-__device__ __forceinline__ int sort_slot(unsigned char* smem, const StageArgs& A, bool need,
-                                         int idx, int ncell) {
-  using S = SmemT<T, R>;
-  constexpr int NT = T::NT, NW = NT / 32, NB = S::NB;
-  static_assert(NB == 32 && NT % 32 == 0 && (NW % 2 == 0), "one lane per bucket, warp pairs");
-  SortSmem<T, R> q(smem);
-  const unsigned full = 0xffffffffu;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  int key = 0;
-  if (need) key = cost_key((int)RHD_LD(A.st, A.cost, idx, ncell));
-  const unsigned m = __match_any_sync(full, key);
-  const int wrank = __popc(m & ((1u << lane) - 1u));
-  if (wrank == 0) RHD_ST(A.st, q.tab, warp * NB + key, NW * NB, __popc(m));
-  __syncthreads();
-  if (warp == 0) {  // lane b: the start of bucket b in each warp
-    int tot = 0;
-    for (int w = 0; w < NW; ++w) tot += q.tab[w * NB + lane];
-    int base = tot;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int v = __shfl_up_sync(full, base, o);
-      if (lane >= o) base += v;
-    }
-    base -= tot;
-    for (int w = 0; w < NW; ++w) {
-      const int c = q.tab[w * NB + lane];
-      q.tab[w * NB + lane] = base;
-      base += c;
-    }
-  }
-  __syncthreads();
-  const int r = (int)RHD_LD(A.st, q.tab, warp * NB + key, NW * NB) + wrank;
-  const int gw = r >> 5;
-  const int tw = gw < NW / 2 ? gw : (3 * NW / 2 - 1) - gw;
-  return tw * 32 + (r & 31);
-}
-
-// this thread's cell (its explicit state; whether it needs a solve) into its
-// sorted slot
-template <class T, typename R>
-__device__ __forceinline__ void stage_slot_put(unsigned char* smem, const StageArgs& A, int slot,
-                                               const double y[8], bool need) {
-  constexpr int NT = T::NT;
-  SortSmem<T, R> q(smem);
-#pragma unroll
-  for (int j = 0; j < 8; ++j) RHD_ST(A.st, q.v, j * NT + slot, 8 * NT, y[j]);
-  RHD_ST(A.st, q.flag, slot, NT, need ? (int)(threadIdx.x << 1) | 1 : 0);
-}
-
-// the cell of slot (this thread's solve): its state, and through src the
-// thread that owns it; clears the bucket counts for the next plane (all
-// threads have read them before the barrier that precedes this call);
-// returns whether the cell needs a solve
-template <class T, typename R>
-__device__ __forceinline__ bool stage_slot_get(unsigned char* smem, const StageArgs& A, int slot,
-                                               double y[8], int& src) {
-  using S = SmemT<T, R>;
-  constexpr int NT = T::NT, NTAB = (NT / 32) * S::NB;
-  SortSmem<T, R> q(smem);
-  for (int i = threadIdx.x; i < NTAB; i += NT) q.tab[i] = 0;
-#pragma unroll
-  for (int j = 0; j < 8; ++j) y[j] = RHD_LD(A.st, q.v, j * NT + slot, 8 * NT);
-  const int f = (int)RHD_LD(A.st, q.flag, slot, NT);
-  src = f >> 1;
-  return (f & 1) != 0;
-}
-
-// the solved cell of slot back into its slot
-template <class T, typename R>
-__device__ __forceinline__ void stage_slot_result(unsigned char* smem, const StageArgs& A,
-                                                  int slot, const double y[8], int code, int nn,
-                                                  int no) {
-  constexpr int NT = T::NT;
-  SortSmem<T, R> q(smem);
-#pragma unroll
-  for (int j = 0; j < 8; ++j) RHD_ST(A.st, q.v, j * NT + slot, 8 * NT, y[j]);
-  RHD_ST(A.st, q.flag, slot, NT, code);
-  RHD_ST(A.st, q.nn, slot, NT, nn);
-  RHD_ST(A.st, q.no, slot, NT, no);
-}
-
-// this thread's own cell, solved, from its sorted slot
-template <class T, typename R>
-__device__ __forceinline__ void stage_slot_take(unsigned char* smem, const StageArgs& A, int slot,
-                                                double y[8], int& code, int& nn, int& no) {
-  constexpr int NT = T::NT;
-  SortSmem<T, R> q(smem);
-#pragma unroll
-  for (int j = 0; j < 8; ++j) y[j] = RHD_LD(A.st, q.v, j * NT + slot, 8 * NT);
-  code = (int)RHD_LD(A.st, q.flag, slot, NT);
-  nn = (int)RHD_LD(A.st, q.nn, slot, NT);
-  no = (int)RHD_LD(A.st, q.no, slot, NT);
-}
-
 struct TileStats {
   int nn_max = 0, no_max = 0;
   unsigned long long nn_sum = 0, no_sum = 0, cnt = 0;
@@ -596,7 +442,13 @@ struct TileStats {
 // reconstruction, closure and HLL fluxes (double for FP64, float for MIXED);
 // the state, the flux differences, the updates and the local solve are double
 // in both.  Every thread of the block must call it (it synchronises).
-template <int STAGE, class T, typename R, bool GEN>
+template <bool MIXED, bool GEN>
+__device__ __noinline__ int local_solve_call(const Physics& ph, double tdt, double rho, double chi,
+                                             double y[8], int& nn, int& no) {
+  return local_solve<MIXED, GEN>(ph, tdt, rho, chi, y, nn, no);
+}
+
+template <int STAGE, class T, typename R, bool GEN, bool CALL = false>
 __device__ __forceinline__ void stage_tile(const StageArgs& A, int x0, int y0, int kbeg,
                                            unsigned char* smem_raw, TileStats& ts) {
   using S = SmemT<T, R>;
@@ -615,13 +467,6 @@ __device__ __forceinline__ void stage_tile(const StageArgs& A, int x0, int y0, i
   if (threadIdx.x == 0) s_chk_status = A.st;
   __syncthreads();
 #endif
-  if constexpr (STAGE != 0) {
-    if (A.cost != nullptr) {  // the sorted solves' bucket counts start at zero
-      SortSmem<T, R> q(smem_raw);
-      for (int i = threadIdx.x; i < (NT / 32) * S::NB; i += NT) q.tab[i] = 0;
-      __syncthreads();
-    }
-  }
   const R chat = (R)ph.chat;
   const double chat6 = ph.chat * (1.0 / 6.0);  // weight of the mixed iso parts
   double* sx = reinterpret_cast<double*>(smem_raw + S::SLOPE_OFF);  // FP64 PLM only
@@ -952,51 +797,19 @@ __device__ __forceinline__ void stage_tile(const StageArgs& A, int x0, int y0, i
           need = !(rk2 && STAGE == 1);
       }
     }
-    if constexpr (STAGE != 0) {
+    if (STAGE != 0 && need) {
       const double tdt = (STAGE == 1 || rk2) ? A.dt : 0.5 * A.dt;
-      // with predicted costs the block's solves run in cost order: each
-      // thread solves the cell of its sorted slot, so that a warp's lanes
-      // take similar numbers of iterations; a cell's arithmetic does not
-      // depend on the lane that runs it, so the results are the same bits
-      const bool sorted = A.cost != nullptr && !(rk2 && STAGE == 1);
-      int myslot = threadIdx.x;
-      bool run = need;
-      if (sorted) {
-        myslot = sort_slot<T, R>(smem_raw, A, need, idx, g.ncell);
-        stage_slot_put<T, R>(smem_raw, A, myslot, y, need);
-        __syncthreads();
-        int src = 0;
-        run = stage_slot_get<T, R>(smem_raw, A, threadIdx.x, y, src);
-        if (run) {  // rho and chi of the slot's cell, as its own thread took them
-          const int sidx = (x0 + src % TX) + g.n[0] * ((y0 + src / TX) + g.n[1] * k);
-          rho = RHD_LD(A.st, A.rho, sidx, g.ncell);
-          chi = RHD_LD(A.st, A.kappa, sidx, g.ncell) * rho;
-        }
-      }
-      int scode = RHD_OK, snn = 0, sno = 0;
-      if (run) {
-        if (GEN && (ph.kappa_P_ratio != 1.0 || ph.kappa_F_ratio != 1.0))
-          scode = local_solve_nongrey<MIXED>(ph, tdt, rho, chi, y, snn, sno);
-        else
-          scode = local_solve<MIXED, GEN>(ph, tdt, rho, chi, y, snn, sno);
-      }
-      if (sorted) {
-        if (run) stage_slot_result<T, R>(smem_raw, A, threadIdx.x, y, scode, snn, sno);
-        __syncthreads();
-        if (need) stage_slot_take<T, R>(smem_raw, A, myslot, y, scode, snn, sno);
-      }
-      if (need) {
-        code = scode;
-        nn = snn;
-        no = sno;
-      }
+      if (GEN && (ph.kappa_P_ratio != 1.0 || ph.kappa_F_ratio != 1.0))
+        code = local_solve_nongrey<MIXED>(ph, tdt, rho, chi, y, nn, no);
+      else if (CALL)
+        code = local_solve_call<MIXED, GEN>(ph, tdt, rho, chi, y, nn, no);
+      else
+        code = local_solve<MIXED, GEN>(ph, tdt, rho, chi, y, nn, no);
     }
     if (col) {
       if (STAGE != 0) {
 #pragma unroll
         for (int q = 0; q < 8; ++q) RHD_ST(A.st, A.yo[q], idx, g.ncell, y[q]);
-        if (A.cost != nullptr && need)
-          RHD_ST(A.st, A.cost, idx, g.ncell, cost_byte(nn, no));
       }
       if (code != RHD_OK) {
         atomicMin(&A.st->fail_key, ((unsigned long long)(A.cell_base + idx) << 8) | (unsigned)code);
