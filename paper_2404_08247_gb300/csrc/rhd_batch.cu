@@ -51,13 +51,13 @@ struct BatchArgs {
   int step;
 };
 
-using Tile1 = TileT<1, 256, 1, 1>;
-using Tile2a = TileT<2, 32, 8, 1>;
-using Tile2b = TileT<2, 64, 4, 1>;
-using Tile2c = TileT<2, 16, 16, 1>;
+using Tile1 = TileT<1, 256, 1>;
+using Tile2a = TileT<2, 32, 8>;
+using Tile2b = TileT<2, 64, 4>;
+using Tile2c = TileT<2, 16, 16>;
 // PPM tiles (kinds 2, 3): the single-grid PPM shapes
-using Tile1P = TileT<1, 256, 1, 1, true>;
-using Tile2P = TileT<2, 32, 8, 1, true>;
+using Tile1P = TileT<1, 256, 1, true>;
+using Tile2P = TileT<2, 32, 8, true>;
 constexpr int kBatchThreads = 256;
 
 // PPMX: the batch holds PPM problems (the kernel then carries both tile kinds)
@@ -107,14 +107,14 @@ __global__ void __launch_bounds__(kBatchThreads, 2) batch_kernel(const BatchArgs
     }
     __syncthreads();
     if (w.kind == 0)
-      stage_tile<STAGE, Tile1, R, GEN, true>(A, w.x0, 0, 0, smem_raw, ts);
+      stage_tile<STAGE, Tile1, R, GEN>(A, w.x0, 0, 0, 1, smem_raw, ts);
     else if (!PPMX || w.kind == 1)
-      stage_tile<STAGE, T2, R, GEN, true>(A, w.x0, w.y0, 0, smem_raw, ts);
+      stage_tile<STAGE, T2, R, GEN>(A, w.x0, w.y0, 0, 1, smem_raw, ts);
     else if constexpr (PPMX) {
       if (w.kind == 2)
-        stage_tile<STAGE, Tile1P, R, true, true>(A, w.x0, 0, 0, smem_raw, ts);
+        stage_tile<STAGE, Tile1P, R, true>(A, w.x0, 0, 0, 1, smem_raw, ts);
       else
-        stage_tile<STAGE, Tile2P, R, true, true>(A, w.x0, w.y0, 0, smem_raw, ts);
+        stage_tile<STAGE, Tile2P, R, true>(A, w.x0, w.y0, 0, 1, smem_raw, ts);
     }
   }
   flush_stats<kBatchThreads>(B.st, ts);

@@ -114,9 +114,9 @@ struct StageArgs {
   // factors of the low slab face (n0 n1)
   const double* halo[2] = {nullptr, nullptr};
   const double* eps_zlo = nullptr;
-  // tile rows skipped along the slowest axis (z in 3-D, y in 2-D, x in 1-D):
-  // a launch over the rows [blk_off, blk_off + grid extent) of that axis
-  int blk_off = 0;
+  // the first cell of the launch along the slowest axis (z in 3-D, y in 2-D, x
+  // in 1-D) and the planes a 3-D block marches through
+  int lo = 0, lz = 1;
 };
 
 // ghost planes a HALO face holds (the widest face stencil: PPM's 3)

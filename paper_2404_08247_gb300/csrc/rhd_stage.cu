@@ -98,19 +98,15 @@ cudaError_t launch_stage(int stage, int precision, const StageArgs& A, cudaStrea
                     : launch_stage_t<2>(precision, A, s, b0, b1);
 }
 
-// Tile rows along the slowest axis, and the cells one row covers (PLM and
-// PPM tiles have the same shape).
+// Tile rows along the slowest axis (the unit of a launch over part of a grid),
+// and the cells one row covers.
 int stage_rows(const Geometry& g) {
-  switch (g.ndim) {
-    case 1: return (g.n[0] + Tile<1>::TX - 1) / Tile<1>::TX;
-    case 2: return (g.n[1] + Tile<2>::TY - 1) / Tile<2>::TY;
-    default: return (g.n[2] + Tile<3>::LZ - 1) / Tile<3>::LZ;
-  }
+  const int w = kRowCells[g.ndim];
+  return (g.n[g.ndim - 1] + w - 1) / w;
 }
 
 long long stage_row_cells(const Geometry& g, int row) {
-  const int ax = g.ndim - 1;
-  const int w = g.ndim == 1 ? Tile<1>::TX : g.ndim == 2 ? Tile<2>::TY : Tile<3>::LZ;
+  const int ax = g.ndim - 1, w = kRowCells[g.ndim];
   long long plane = 1;
   for (int d = 0; d < ax; ++d) plane *= g.n[d];
   const int lo = row * w, hi = std::min(g.n[ax], lo + w);

@@ -20,45 +20,42 @@
 
 namespace rhd {
 
-// A tile: TX x TY threads (one per cell of a plane), LZ planes per block in
-// 3-D.  PPM: piecewise parabolic faces (else PLM).  HX, HY: halo widths; NPL:
-// planes kept in the shared-memory ring.
-template <int NDIM_, int TX_, int TY_, int LZ_, bool PPM_ = false>
+// A tile: TX x TY threads, one per cell of a plane.  PPM: piecewise parabolic
+// faces (else PLM).  HX, HY: halo widths; NPL: planes kept in the
+// shared-memory ring.
+template <int NDIM_, int TX_, int TY_, bool PPM_ = false>
 struct TileT {
-  static constexpr int NDIM = NDIM_, TX = TX_, TY = TY_, LZ = LZ_;
+  static constexpr int NDIM = NDIM_, TX = TX_, TY = TY_;
   static constexpr bool PPM = PPM_;
   static constexpr int HX = PPM ? 3 : 2, HY = NDIM >= 2 ? HX : 0;
   static constexpr int NPL = NDIM == 3 ? 4 : 1;
   static constexpr int NT = TX * TY;
 };
 
-template <int NDIM>
-struct DefaultTileOf;
-// 3-D: 8 planes per block.  Longer z-chunks load fewer halo planes, but the
-// per-block cost varies with the local physics (iteration counts), and short
-// chunks balance the SMs better (256^3: 8 planes 2.6 % faster than 32).
-// Build-time shape of the 3-D tile (rows TY of 32 cells, LZ planes per
-// block) and the blocks per SM its stage kernels are compiled for.
-#ifndef RHD_TILE3_TY
-#define RHD_TILE3_TY 8
-#endif
-#ifndef RHD_TILE3_LZ
-#define RHD_TILE3_LZ 8
-#endif
+// The tiles of the grid kernels (shapes and the planes a 3-D block marches
+// through: TilePlan, rhd_stage.cuh).  SMALL: one or two warps, for grids that
+// leave SMs idle with the large tile; rows a launch over part of a grid counts
+// in (the large tile's width along the slowest axis, 8 planes in 3-D) are
+// whole numbers of small ones.
+constexpr int kRowCells[4] = {0, 256, 8, 8};
+template <int NDIM, bool SMALL>
+struct TileShape;
 template <>
-struct DefaultTileOf<3> { using type = TileT<3, 32, RHD_TILE3_TY, RHD_TILE3_LZ>; };
+struct TileShape<3, false> { static constexpr int TX = 32, TY = 8; };
 template <>
-struct DefaultTileOf<2> { using type = TileT<2, 32, 8, 1>; };
+struct TileShape<2, false> { static constexpr int TX = 32, TY = 8; };
 template <>
-struct DefaultTileOf<1> { using type = TileT<1, 256, 1, 1>; };
-template <int NDIM>
-using Tile = typename DefaultTileOf<NDIM>::type;
-
-// PPM tiles: the same shapes with the wider halo (3-D, FP64: 86 KB of
-// shared memory, two blocks per SM).
-template <int NDIM>
-using TilePPM = TileT<NDIM, DefaultTileOf<NDIM>::type::TX, DefaultTileOf<NDIM>::type::TY,
-                      DefaultTileOf<NDIM>::type::LZ, true>;
+struct TileShape<1, false> { static constexpr int TX = 256, TY = 1; };
+template <>
+struct TileShape<3, true> { static constexpr int TX = 16, TY = 4; };
+template <>
+struct TileShape<2, true> { static constexpr int TX = 16, TY = 4; };
+template <>
+struct TileShape<1, true> { static constexpr int TX = 32, TY = 1; };
+// PPM tiles: the same shapes with the wider halo (3-D, FP64, large: 86 KB of
+// shared memory, two blocks per SM)
+template <int NDIM, bool PPM, bool SMALL>
+using TileOf = TileT<NDIM, TileShape<NDIM, SMALL>::TX, TileShape<NDIM, SMALL>::TY, PPM>;
 
 // ring slot of plane p (p >= -3)
 template <class T>
@@ -434,22 +431,25 @@ struct TileStats {
   unsigned long long nn_sum = 0, no_sum = 0, cnt = 0;
 };
 
-// One tile of one stage (STAGE 1, 2, or 0 = transport rates only; GEN: with
-// the general physics, RK2-SSP, a temperature-dependent opacity and inflow
-// faces, which the default physics compiles out): the block
-// of T::NT threads owns the cells x0 + [0, TX) x y0 + [0, TY) x planes
-// [kbeg, kbeg + LZ) of the grid described by A.  R: precision of
-// reconstruction, closure and HLL fluxes (double for FP64, float for MIXED);
-// the state, the flux differences, the updates and the local solve are double
-// in both.  Every thread of the block must call it (it synchronises).
+// local_solve as a call: its registers are then allocated apart from the
+// tile's (inlined, the batched kernel spilled 744 bytes a thread, now 196), and
+// the kernels of a unit share one copy.
 template <bool MIXED, bool GEN>
 __device__ __noinline__ int local_solve_call(const Physics& ph, double tdt, double rho, double chi,
                                              double y[8], int& nn, int& no) {
   return local_solve<MIXED, GEN>(ph, tdt, rho, chi, y, nn, no);
 }
 
-template <int STAGE, class T, typename R, bool GEN, bool CALL = false>
-__device__ __forceinline__ void stage_tile(const StageArgs& A, int x0, int y0, int kbeg,
+// One tile of one stage (STAGE 1, 2, or 0 = transport rates only; GEN: with
+// the general physics, RK2-SSP, a temperature-dependent opacity and inflow
+// faces, which the default physics compiles out): the block
+// of T::NT threads owns the cells x0 + [0, TX) x y0 + [0, TY) x planes
+// [kbeg, kend) of the grid described by A.  R: precision of
+// reconstruction, closure and HLL fluxes (double for FP64, float for MIXED);
+// the state, the flux differences, the updates and the local solve are double
+// in both.  Every thread of the block must call it (it synchronises).
+template <int STAGE, class T, typename R, bool GEN>
+__device__ __forceinline__ void stage_tile(const StageArgs& A, int x0, int y0, int kbeg, int kend,
                                            unsigned char* smem_raw, TileStats& ts) {
   using S = SmemT<T, R>;
   constexpr int NDIM = T::NDIM;
@@ -476,7 +476,6 @@ __device__ __forceinline__ void stage_tile(const StageArgs& A, int x0, int y0, i
   const bool col = ix < g.n[0] && (NDIM < 2 || iy < g.n[1]);
   const int cy = NDIM >= 2 ? min(iy, g.n[1] - 1) : 0;  // clamped row of the column
   const int cx = min(ix, g.n[0] - 1);
-  const int kend = min(kbeg + T::LZ, g.n[2]);
   const int own = (tx + T::HX) + (ty + T::HY) * S::PW;  // own cell in a plane
 
   bool zbad = false;
@@ -801,10 +800,8 @@ __device__ __forceinline__ void stage_tile(const StageArgs& A, int x0, int y0, i
       const double tdt = (STAGE == 1 || rk2) ? A.dt : 0.5 * A.dt;
       if (GEN && (ph.kappa_P_ratio != 1.0 || ph.kappa_F_ratio != 1.0))
         code = local_solve_nongrey<MIXED>(ph, tdt, rho, chi, y, nn, no);
-      else if (CALL)
-        code = local_solve_call<MIXED, GEN>(ph, tdt, rho, chi, y, nn, no);
       else
-        code = local_solve<MIXED, GEN>(ph, tdt, rho, chi, y, nn, no);
+        code = local_solve_call<MIXED, GEN>(ph, tdt, rho, chi, y, nn, no);
     }
     if (col) {
       if (STAGE != 0) {
