@@ -274,7 +274,10 @@ __device__ __forceinline__ double half_slope<double>(double um, double u0, doubl
 // = (u0 + up)/2 - (h1 - h0)/3; it lies between u0 and up.
 template <typename R>
 __device__ __forceinline__ R ppm_interface(R u0, R up, R h0, R h1) {
-  return R(0.5) * (u0 + up) - (h1 - h0) * R(1.0 / 3.0);
+  if constexpr (sizeof(R) == sizeof(double))
+    return fma(sub(h0, h1), 1.0 / 3.0, half_of(add(u0, up)));
+  else
+    return R(0.5) * (u0 + up) - (h1 - h0) * R(1.0 / 3.0);
 }
 
 // Their monotonicity constraint (eq. 1.10) on the edge values (l, r) of a
@@ -295,8 +298,8 @@ __device__ __forceinline__ R ppm_edge(R u0, R l, R r) {
   return LEFT ? u0 - copysign(m, a) : u0 + copysign(m, a);
 }
 
-// double: the sign tests and minima on the integer pipe (non-negative doubles
-// order as their bit patterns; 2|b| = |b + b| exactly)
+// double: the sign tests, the minima and 2|b| on the integer pipe (non-negative
+// doubles order as their bit patterns)
 template <bool LEFT>
 __device__ __forceinline__ double ppm_edge_d(double u0, double l, double r) {
   const double dl = u0 - l, dr = r - u0;
@@ -304,7 +307,8 @@ __device__ __forceinline__ double ppm_edge_d(double u0, double l, double r) {
   const long long ba = dbits(a), bb = dbits(b);
   const long long ma = ba & kMag, mb = bb & kMag;
   const bool mono = ((ba ^ bb) >= 0) & (ma != 0) & (mb != 0);
-  const long long m = min(ma, abs_bits(b + b));
+  const bool plain = mb >= (1ll << 52) && mb < kInfBits - (1ll << 52);
+  const long long m = min(ma, plain ? mb + (1ll << 52) : abs_bits(b + b));
   const double s = __longlong_as_double(mono ? (m | (ba & ~kMag)) : 0ll);
   return LEFT ? u0 - s : u0 + s;
 }

@@ -77,7 +77,20 @@ struct SmemT {
   static constexpr int FY = T::NDIM >= 2 ? 4 * (T::TY + 1) * T::TX : 0;
   // PPM z march: each thread's carried right edge and interface value (kept
   // in shared memory: in registers they push the FP64 kernel past its budget)
-  static constexpr int CZ = (T::PPM && T::NDIM == 3) ? 12 * T::NT : 0;
+  // (12 values: the Colella-Sekora march carries a second difference as well)
+  //
+  // FP64 PPM: the interface values of a plane along x, then those along y, in
+  // the same place: the faces -1 .. TX + 1 of the tile's rows, so that each is
+  // computed once and not for the three faces that read it.  They share the
+  // Colella-Sekora march's second differences' place (which recomputes its
+  // interface values): with that, two blocks of the 3-D tile fit an SM.
+  static constexpr bool IFACE = T::PPM && sizeof(R) == sizeof(double);
+  static constexpr int AX = IFACE ? T::TY * (T::TX + 3) : 0;  // per field
+  static constexpr int AY = IFACE && T::NDIM >= 2 ? (T::TY + 3) * T::TX : 0;
+  static constexpr int CZ0 = (T::PPM && T::NDIM == 3) ? 8 * T::NT : 0;
+  static constexpr int CZ2 = (T::PPM && T::NDIM == 3) ? 4 * T::NT : 0;
+  static constexpr int AXY = 4 * (AX > AY ? AX : AY);
+  static constexpr int CZ = CZ0 + (CZ2 > AXY ? CZ2 : AXY);
   // mixed precision: the isotropic part of each x-/y-face's normal momentum
   // flux in double (hll_states_mixed), after the R arrays (16-byte aligned)
   static constexpr bool ISO = sizeof(R) == sizeof(float);
@@ -334,13 +347,25 @@ __device__ __forceinline__ void ppm_states(const R u[6][4], R L[4], R Rr[4], boo
 
 // flux through the face between plane cells c - st and c (stride st); cs:
 // PPM tiles with the Colella-Sekora limiter; iso: see face_hll
-// (sl, sr: the half slopes of cells c - st and c, field q at q * sn; FP64 PLM)
+// (FP64 PLM: sl, sr are the half slopes of cells c - st and c, field q at q *
+// sn.  FP64 PPM with CW84's limiter: sl the interface value at the face before,
+// sr that of this face, sr + (sr - sl) that of the next)
 template <class T, typename R>
 __device__ __forceinline__ bool plane_face(const R* pl, int c, int st, int d, R eps, R chat,
                                            int closure, R out[4], double& iso, const double* sl,
                                            const double* sr, int sn, bool cs = false) {
   R L[4], Rr[4];
-  if constexpr (T::PPM) {
+  if (SmemT<T, R>::IFACE && !cs) {
+    R a[4], b[4];
+    cell_of<T, R>(pl, c - st, a);
+    cell_of<T, R>(pl, c, b);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const R a0 = (R)sl[q * sn], a1 = (R)sr[q * sn], a2 = (R)sr[q * sn + (sr - sl)];
+      L[q] = ppm_edge_of<false>(a[q], a0, a1);
+      Rr[q] = ppm_edge_of<true>(b[q], a1, a2);
+    }
+  } else if constexpr (T::PPM) {
     R u[6][4];
 #pragma unroll
     for (int o = 0; o < 6; ++o) cell_of<T, R>(pl, c + (o - 3) * st, u[o]);
@@ -489,6 +514,7 @@ __device__ __forceinline__ void stage_tile(const StageArgs& A, int x0, int y0, i
   R* rz = fys + S::FY + threadIdx.x;       // rz[q * NT]: right edge of cell k
   R* az = rz + 4 * NT;                      // az[q * NT]: interface value a(k+1/2)
   R* dz = az + 4 * NT;                      // dz[q * NT]: second difference of cell k
+  double* ia = reinterpret_cast<double*>(fys + S::FY + S::CZ0);  // FP64 PPM interface values
   const bool cs = T::PPM && ph.reconstruction == RHD_RECON_PPM_CS;
   if constexpr (NDIM == 3 && T::PPM) {
     R u[6][4];
@@ -681,6 +707,26 @@ __device__ __forceinline__ void stage_tile(const StageArgs& A, int x0, int y0, i
       __syncthreads();
     }
 
+    // ---- FP64 PPM: the interface value between cells c - st and c
+    auto interface = [&](int c, int st, double* out, int sn) {
+      if constexpr (S::IFACE) {
+        double u[4][4];
+#pragma unroll
+        for (int o = 0; o < 4; ++o) cell_of<T, R>(pl, c + (o - 2) * st, u[o]);
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          out[q * sn] = ppm_interface(u[1][q], u[2][q], half_slope(u[0][q], u[1][q], u[2][q]),
+                                      half_slope(u[1][q], u[2][q], u[3][q]));
+      }
+    };
+    if (S::IFACE && !cs) {
+      for (int i = threadIdx.x; i < S::AX; i += NT) {
+        const int j = i % (TX + 3), r = i / (TX + 3);
+        interface(j - 1 + T::HX + (r + T::HY) * S::PW, 1, ia + i, S::AX);
+      }
+      __syncthreads();
+    }
+
     // ---- x-faces of plane k: face f lies between tile cells fi-1 and fi
     for (int f = threadIdx.x; f < (TX + 1) * TY; f += NT) {
       int fi = f % (TX + 1), fj = f / (TX + 1);
@@ -691,8 +737,9 @@ __device__ __forceinline__ void stage_tile(const StageArgs& A, int x0, int y0, i
       R eps = real ? (R)face_eps(A, 0, xl, yr, k) : R(1);
       R out[4];
       double iso;
-      const double* sl = sx + fj * (TX + 2) + fi;
-      if (!plane_face<T, R>(pl, c, 1, 0, eps, chat, ph.closure, out, iso, sl, sl + 1, S::SX, cs) &&
+      const double* sl = S::IFACE ? ia + fj * (TX + 3) + fi : sx + fj * (TX + 2) + fi;
+      if (!plane_face<T, R>(pl, c, 1, 0, eps, chat, ph.closure, out, iso, sl, sl + 1,
+                            S::IFACE ? S::AX : S::SX, cs) &&
           real) {
         // a face with E <= 0 poisons both neighbours' fluxes
 #pragma unroll
@@ -704,6 +751,14 @@ __device__ __forceinline__ void stage_tile(const StageArgs& A, int x0, int y0, i
     }
     // ---- y-faces of plane k: face f lies between rows fj-1 and fj
     if (NDIM >= 2) {
+      if (S::IFACE && !cs) {
+        __syncthreads();  // every x-face has read its interface values
+        for (int i = threadIdx.x; i < S::AY; i += NT) {
+          const int x = i % TX, j = i / TX;
+          interface(x + T::HX + (j - 1 + T::HY) * S::PW, S::PW, ia + i, S::AY);
+        }
+        __syncthreads();
+      }
       for (int f = threadIdx.x; f < TX * (TY + 1); f += NT) {
         int fi = f % TX, fj = f / TX;
         int c = fi + T::HX + (fj + T::HY) * S::PW;
@@ -712,9 +767,9 @@ __device__ __forceinline__ void stage_tile(const StageArgs& A, int x0, int y0, i
         R eps = real ? (R)face_eps(A, 1, xr, yl, k) : R(1);
         R out[4];
         double iso;
-        const double* sl = sy + fj * TX + fi;
-        if (!plane_face<T, R>(pl, c, S::PW, 1, eps, chat, ph.closure, out, iso, sl, sl + TX, S::SY,
-                              cs) &&
+        const double* sl = (S::IFACE ? ia : sy) + fj * TX + fi;
+        if (!plane_face<T, R>(pl, c, S::PW, 1, eps, chat, ph.closure, out, iso, sl, sl + TX,
+                              S::IFACE ? S::AY : S::SY, cs) &&
             real) {
 #pragma unroll
           for (int q = 0; q < 4; ++q) out[q] = (R)__longlong_as_double(0x7ff8000000000000ll);
