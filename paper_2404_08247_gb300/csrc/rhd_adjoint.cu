@@ -44,27 +44,28 @@ __device__ __forceinline__ long long face_index(const Geometry& g, int d, int x,
   return x + (long long)n0 * (y + (long long)n1 * z);
 }
 
-// Half PLM slope (monotonised-central limiter) and its gradient with respect to
-// (u_-, u_0, u_+) on the active branch; zero at an extremum.  Signs and the
+// Half PLM slope (monotonised-central limiter) and the candidate it selects:
+// 0 none (extremum), 1 u_0 - u_-, 2 u_+ - u_0, 3 (u_+ - u_-)/4.  Signs and the
 // minimum are taken on the integer pipe, as in the forward half_slope.
-__device__ __forceinline__ double half_slope_vjp(double um, double u0, double up, double& gm,
-                                                 double& g0, double& gp) {
+__device__ __forceinline__ double half_slope_branch(double um, double u0, double up, int& br) {
   double dm = u0 - um, dp = up - u0;
-  double q = 0.25 * (dm + dp);
   long long bm = dbits(dm), bp = dbits(dp);
-  long long am = bm & kMag, ap = bp & kMag, aq = abs_bits(q);
-  gm = g0 = gp = 0.0;
+  long long am = bm & kMag, ap = bp & kMag, aq = quarter_bits(dm + dp);
+  br = 0;
   if (!(((bm ^ bp) >= 0) & (am != 0) & (ap != 0))) return 0.0;
   long long m = min(min(am, ap), aq);
-  // the selected candidate, as a signed linear form in (um, u0, up)
-  if (m == am) {
-    gm = -1.0; g0 = 1.0;
-  } else if (m == ap) {
-    g0 = -1.0; gp = 1.0;
-  } else {
-    gm = -0.25; gp = 0.25;
-  }
+  br = m == am ? 1 : m == ap ? 2 : 3;
   return __longlong_as_double(m | (bm & ~kMag));
+}
+
+// Reverse of it: the slope's cotangent s onto (u_-, u_0, u_+), whose partials
+// are 0, +-1 or +-1/4 by the branch, so that nothing is multiplied.
+__device__ __forceinline__ void half_slope_vjp(int br, double s, double& gm, double& g0,
+                                               double& gp) {
+  const double q = 0.25 * s;
+  gm = br == 1 ? -s : br == 3 ? -q : 0.0;
+  g0 = br == 1 ? s : br == 2 ? -s : 0.0;
+  gp = br == 2 ? s : br == 3 ? q : 0.0;
 }
 
 // One face state after the free-streaming rescale, with the closure
@@ -77,16 +78,25 @@ struct FaceState {
   double P[3];  // row d of P
 };
 
+// (with h = s/2 = sqrt(E^2 - 3/4 |Ft|^2) as in the forward face_side; a flux
+// scaled back has |Ft| = E)
 __device__ __forceinline__ void face_state(int d, int closure, double E, const double Fin[3],
                                            FaceState& s) {
   s.E = E;
-  s.n2 = Fin[0] * Fin[0] + Fin[1] * Fin[1] + Fin[2] * Fin[2];
-  s.resc = lt_nn(E * E, s.n2);
-  double sc = s.resc ? E * rsqrt_pos(s.n2) : 1.0;
+  s.n2 = dot3(Fin, Fin);
+  const double E2 = E * E;
+  s.resc = lt_nn(E2, s.n2);
 #pragma unroll
   for (int j = 0; j < 3; ++j) {
     s.Fin[j] = Fin[j];
-    s.F[j] = Fin[j] * sc;
+    s.F[j] = Fin[j];
+  }
+  double F2 = s.n2;
+  if (s.resc) {
+    const double sc = E * rsqrt_pos(s.n2);
+#pragma unroll
+    for (int j = 0; j < 3; ++j) s.F[j] = Fin[j] * sc;
+    F2 = E2;
   }
   if (closure == RHD_CLOSURE_EDDINGTON) {
     s.ha = E * (1.0 / 3.0);
@@ -94,28 +104,17 @@ __device__ __forceinline__ void face_state(int d, int closure, double E, const d
     s.ha_E = 1.0 / 3.0;
     s.ha_F2 = s.hb_E = s.hb_F2 = 0.0;
   } else {
-    double F2 = s.F[0] * s.F[0] + s.F[1] * s.F[1] + s.F[2] * s.F[2];
-    if (lt_nn(E * E, F2)) {  // only through rounding of the rescale
-      double iF2 = rcp_pos(F2);
-      s.ha = 0.0;
-      s.hb = E * iF2;
-      s.ha_E = s.ha_F2 = 0.0;
-      s.hb_E = iF2;
-      s.hb_F2 = -E * iF2 * iF2;
-    } else {
-      // s = sqrt(4E^2 - 3F2), ha = (s - E)/3, hb = 3/(2E + s)
-      double x = 4.0 * E * E - 3.0 * F2;
-      double ir = rsqrt_pos(x);
-      double r = x * ir;
-      s.ha = (r - E) * (1.0 / 3.0);
-      s.hb = 3.0 * rcp_pos(2.0 * E + r);
-      double r_E = 4.0 * E * ir, r_F2 = -1.5 * ir;
-      s.ha_E = (r_E - 1.0) * (1.0 / 3.0);
-      s.ha_F2 = r_F2 * (1.0 / 3.0);
-      double hb2 = s.hb * s.hb * (1.0 / 3.0);
-      s.hb_E = -hb2 * (2.0 + r_E);
-      s.hb_F2 = -hb2 * r_F2;
-    }
+    // ha = (2h - E)/3, hb = 3/2/(E + h)
+    const double x = fma(-0.75, F2, E2);
+    const double ih = rsqrt_pos(x), h = x * ih;
+    const double w = rcp_pos(E + h), hb2 = 0.75 * w * w;
+    const double h2E = 2.0 * E * ih;  // d(2h)/dE
+    s.ha = fma(2.0, h, -E) * (1.0 / 3.0);
+    s.hb = 1.5 * w;
+    s.ha_E = (h2E - 1.0) * (1.0 / 3.0);
+    s.ha_F2 = -0.25 * ih;
+    s.hb_E = -hb2 * (2.0 + h2E);
+    s.hb_F2 = hb2 * 0.75 * ih;
   }
   double t = s.hb * s.F[d];
 #pragma unroll
@@ -149,16 +148,16 @@ __device__ __forceinline__ void face_state_vjp(int d, const FaceState& s, const 
   }
 }
 
-// d/dtau of the optical-depth factor (1 - exp(-tau))/tau.  Below tau = 0.05 the
-// closed form cancels; there its Taylor series sum_k (-1)^k k tau^(k-1)/(k+1)!
-// is used through tau^5 (truncation < 1e-14 relative).
-__device__ __forceinline__ double tau_factor_deriv(double tau) {
+// d/dtau of the optical-depth factor eps = (1 - exp(-tau))/tau: (1 - eps)/tau -
+// eps.  Below tau = 0.05 the difference cancels; there its Taylor series
+// sum_k (-1)^k k tau^(k-1)/(k+1)! is used through tau^5 (truncation < 1e-14
+// relative).
+__device__ __forceinline__ double tau_factor_deriv(double tau, double eps) {
   if (tau < 0.05) {
     return -0.5 + tau * (1.0 / 3.0 + tau * (-0.125 + tau * (1.0 / 30.0 +
            tau * (-1.0 / 144.0 + tau * (1.0 / 840.0 - tau * (1.0 / 5760.0))))));
   }
-  double e = exp(-tau);
-  return (e * (1.0 + tau) - 1.0) / (tau * tau);
+  return fma(1.0 - eps, rcp_pos(tau), -eps);
 }
 
 struct FaceArgs {
@@ -168,7 +167,8 @@ struct FaceArgs {
   const double* kappa;
   const double* y[4];    // state whose transport is differentiated: E, Fx, Fy, Fz
   const double* cot[4];  // cotangent of the stage target: E, Fx, Fy, Fz
-  double alpha;          // the stage weight of s (dt or dt/2)
+  const double* eps[3];  // TAU mode: the forward's factors of the +d faces
+  double wE[3], wF[3];   // cotangent weights: chat/2 theta dt/dx_d, times c for F
   double* fp;            // face partials, FP_SLOTS per face, slot-major per axis
   long long off[3];      // start of axis d in fp
   long long nface[3];
@@ -210,24 +210,23 @@ __device__ __forceinline__ void face_vjp(const FaceArgs& A, long long fidx) {
     for (int j = 0; j < 3; ++j) u[p][1 + j] = __ldg(A.y[1 + j] + idx[p]) * inv_c;
     if (flip) u[p][1 + d] = -u[p][1 + d];
   }
-  // face cotangent: the face flux enters rate(b) with +1/dx and rate(a) with
-  // -1/dx; rates of F are c times those of Ft; ghost cells carry no rate
+  // face cotangent (of the flux in units of chat/2): the face flux enters the
+  // update of b with the weight and that of a with its negative; ghost cells
+  // carry no update
   double ob[4];
-  {
-    double s = A.alpha * g.inv_dx[d];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      double ub = ghost[2] ? 0.0 : __ldg(A.cot[q] + idx[2]);
-      double ua = ghost[1] ? 0.0 : __ldg(A.cot[q] + idx[1]);
-      ob[q] = (ub - ua) * s * (q == 0 ? 1.0 : A.ph.c);
-    }
-  }
-  // ---- forward: reconstruction, closure, speeds ----
-  double L[4], R[4], gl[4][3], gr[4][3];
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
-    L[q] = u[1][q] + half_slope_vjp(u[0][q], u[1][q], u[2][q], gl[q][0], gl[q][1], gl[q][2]);
-    R[q] = u[2][q] - half_slope_vjp(u[1][q], u[2][q], u[3][q], gr[q][0], gr[q][1], gr[q][2]);
+    double ub = ghost[2] ? 0.0 : __ldg(A.cot[q] + idx[2]);
+    double ua = ghost[1] ? 0.0 : __ldg(A.cot[q] + idx[1]);
+    ob[q] = (ub - ua) * (q == 0 ? A.wE[d] : A.wF[d]);
+  }
+  // ---- forward: reconstruction, closure, speeds ----
+  double L[4], R[4];
+  int bl[4], br[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    L[q] = u[1][q] + half_slope_branch(u[0][q], u[1][q], u[2][q], bl[q]);
+    R[q] = u[2][q] - half_slope_branch(u[1][q], u[2][q], u[3][q], br[q]);
   }
   FaceState sl, sr;
   face_state(d, A.ph.closure, L[0], &L[1], sl);
@@ -239,41 +238,41 @@ __device__ __forceinline__ void face_vjp(const FaceArgs& A, long long fidx) {
     den = sr.E;
     side = 1;
   }
-  if (lt_nn(3.0 * num, den)) side = -1;
-  const double chat = A.ph.chat;
-  // S = chat sqrt(num/den) = chat num / sqrt(num den)
-  double rq = side < 0 ? 0.0 : rsqrt_pos(num * den);
-  double S = side < 0 ? chat * sqrt(1.0 / 3.0) : chat * num * rq;
+  if (lt_nn(3.0 * num, den)) {
+    num = 1.0;
+    den = 3.0;
+    side = -1;
+  }
+  // S/chat = sqrt(num/den) = num/sqrt(num den)
+  const double rq = rsqrt_pos(num * den);
+  const double S = num * rq;
   double eps = 1.0, tau = 0.0;
-  bool tau_mode = A.ph.hll_mode == RHD_HLL_TAU;
+  const bool tau_mode = A.ph.hll_mode == RHD_HLL_TAU;
   if (tau_mode) {
     tau = 0.5 * (__ldg(A.kappa + idx[1]) * __ldg(A.rho + idx[1]) +
                  __ldg(A.kappa + idx[2]) * __ldg(A.rho + idx[2])) * g.dx[d];
-    eps = tau_factor(tau);
+    eps = ghost[1] ? tau_factor(tau) : __ldg(A.eps[d] + idx[1]);
   }
   // ---- reverse: HLL ----
-  const double hc = 0.5 * chat, hS = 0.5 * S;
-  double dE = sr.E - sl.E;
-  double gEL = eps * hS * ob[0], gER = -gEL;
+  const double dE = sr.E - sl.E;
+  double gEL = eps * S * ob[0], gER = -gEL;
   double gFL[3] = {0.0, 0.0, 0.0}, gFR[3] = {0.0, 0.0, 0.0};
   double gPL[3], gPR[3];
-  gFL[d] = hc * ob[0];
-  gFR[d] = hc * ob[0];
-  double geps = -hS * dE * ob[0];
-  double ghS = -eps * dE * ob[0];
+  gFL[d] = ob[0];
+  gFR[d] = ob[0];
+  const double geps = -S * dE * ob[0];
+  double gS = -eps * dE * ob[0];
 #pragma unroll
   for (int j = 0; j < 3; ++j) {
-    gPL[j] = hc * ob[1 + j];
-    gPR[j] = hc * ob[1 + j];
-    gFR[j] -= hS * ob[1 + j];
-    gFL[j] += hS * ob[1 + j];
-    ghS -= (sr.F[j] - sl.F[j]) * ob[1 + j];
+    gPL[j] = ob[1 + j];
+    gPR[j] = ob[1 + j];
+    gFR[j] -= S * ob[1 + j];
+    gFL[j] += S * ob[1 + j];
+    gS -= (sr.F[j] - sl.F[j]) * ob[1 + j];
   }
   if (side >= 0) {
-    // S = chat sqrt(num/den): dS/d(num/den) = chat^2 / (2 S), 1/S = den rq / chat
-    double gx = 0.25 * ghS * chat * den * rq;
-    double iden = rcp_pos(den);
-    double gnum = gx * iden, gden = -gx * num * iden * iden;
+    // dS/dnum = 1/(2 sqrt(num den)), dS/dden = -S^2 of that
+    const double gnum = 0.5 * gS * rq, gden = -gnum * S * S;
     if (side == 0) {
       gPL[d] += gnum;
       gEL += gden;
@@ -284,36 +283,35 @@ __device__ __forceinline__ void face_vjp(const FaceArgs& A, long long fidx) {
   }
   face_state_vjp(d, sl, gPL, gEL, gFL);
   face_state_vjp(d, sr, gPR, gER, gFR);
-  // ---- reverse: reconstruction ----
+  // ---- reverse: reconstruction, for E and the physical F (Ft = F/c) ----
   double gq[4][4];
-#pragma unroll
-  for (int p = 0; p < 4; ++p)
-#pragma unroll
-    for (int q = 0; q < 4; ++q) gq[p][q] = 0.0;
   {
-    double gLq[4] = {gEL, gFL[0], gFL[1], gFL[2]};
-    double gRq[4] = {gER, gFR[0], gFR[1], gFR[2]};
+    const double gLq[4] = {gEL, gFL[0] * inv_c, gFL[1] * inv_c, gFL[2] * inv_c};
+    const double gRq[4] = {gER, gFR[0] * inv_c, gFR[1] * inv_c, gFR[2] * inv_c};
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-      gq[0][q] += gLq[q] * gl[q][0];
-      gq[1][q] += gLq[q] * (1.0 + gl[q][1]) - gRq[q] * gr[q][0];
-      gq[2][q] += gLq[q] * gl[q][2] + gRq[q] * (1.0 - gr[q][1]);
-      gq[3][q] -= gRq[q] * gr[q][2];
+      double lm, l0, lp, rm, r0, rp;
+      half_slope_vjp(bl[q], gLq[q], lm, l0, lp);
+      half_slope_vjp(br[q], -gRq[q], rm, r0, rp);
+      gq[0][q] = lm;
+      gq[1][q] = (gLq[q] + l0) + rm;
+      gq[2][q] = (gRq[q] + r0) + lp;
+      gq[3][q] = rp;
     }
   }
-  // store: d/dE and d/dF (physical F: Ft = F/c), not yet mirrored
+  // store, not yet mirrored
   double* out = A.fp + A.off[d] + fidx;
   const long long NF = A.nface[d];
 #pragma unroll
   for (int p = 0; p < 4; ++p) {
     out[(4 * p) * NF] = gq[p][0];
 #pragma unroll
-    for (int j = 0; j < 3; ++j) out[(4 * p + 1 + j) * NF] = gq[p][1 + j] * inv_c;
+    for (int j = 0; j < 3; ++j) out[(4 * p + 1 + j) * NF] = gq[p][1 + j];
   }
   double ka = 0.0, kb = 0.0;
   if (tau_mode) {
     // tau = (chi_a + chi_b) dx/2, chi = kappa rho
-    double gt = geps * tau_factor_deriv(tau) * 0.5 * g.dx[d];
+    double gt = geps * tau_factor_deriv(tau, eps) * 0.5 * g.dx[d];
     ka = gt * __ldg(A.rho + idx[1]);
     kb = gt * __ldg(A.rho + idx[2]);
   }
@@ -382,77 +380,40 @@ __device__ __forceinline__ void gather_axis(const Geometry& g, const double* fp,
 
 // ---------------------------------------------------------- local solve
 
-// Solve M x = b for a 5 x 5 M (row-major, destroyed) by Gaussian elimination
-// with partial pivoting; rows are swapped with compile-time indices only.
-__device__ __forceinline__ bool solve5(double M[5][5], double b[5]) {
-  double ipiv[5];
-#pragma unroll
-  for (int col = 0; col < 5; ++col) {
-    // pivot: the largest |M[r][col]|, r >= col, moved into row col
-#pragma unroll
-    for (int r = col + 1; r < 5; ++r) {
-      if (abs_bits(M[col][col]) < abs_bits(M[r][col])) {
-#pragma unroll
-        for (int k = 0; k < 5; ++k) {
-          double t = M[col][k];
-          M[col][k] = M[r][k];
-          M[r][k] = t;
-        }
-        double t = b[col];
-        b[col] = b[r];
-        b[r] = t;
-      }
-    }
-    const long long pb = dbits(M[col][col]);
-    if ((pb & kMag) == 0 || (pb & kMag) >= kInfBits) return false;
-    // 1/pivot with the pivot's sign
-    const double inv = __longlong_as_double(
-        dbits(rcp_pos(__longlong_as_double(pb & kMag))) | (pb & ~kMag));
-    ipiv[col] = inv;
-#pragma unroll
-    for (int r = col + 1; r < 5; ++r) {
-      double f = M[r][col] * inv;
-#pragma unroll
-      for (int k = col + 1; k < 5; ++k) M[r][k] -= f * M[col][k];
-      b[r] -= f * b[col];
-    }
-  }
-#pragma unroll
-  for (int i = 4; i >= 0; --i) {
-    double s = b[i];
-#pragma unroll
-    for (int k = i + 1; k < 5; ++k) s -= M[i][k] * b[k];
-    b[i] = s * ipiv[i];
-  }
-  return true;
-}
-
 // Adjoint of one converged local solve with output y (Egas, m, E, F) and
 // stage weight theta (tdt = theta dt).  ybar: cotangent of the output; on exit
 // yin: cotangent of the input state; chibar: dL/dchi.  Returns false if the
 // Jacobian of the converged system is singular.
+//
+// (dr/dx)^T lambda = xbar is solved by its structure instead of a 5 x 5
+// elimination.  The rows r_G + (c/chat) r_E = Egas - Egas(t) + (c/chat)(E -
+// E(t)) and r_E leave mu0 and mu1 (lambda_G = mu0, lambda_E = (c/chat) mu0 +
+// mu1) explicit in V = v.mu and U = Ft.mu, mu the flux rows' multipliers, whose
+// own block is al I plus products of v and Ft:
+//   d mu1 = x1 - (c/chat) x0 - (bv - (c/chat) a0) V - bu U,
+//   al mu = x - v (vv V + uv U - ev mu1) - Ft (vu V + uu U - eu mu1),
+// and its products with v and Ft are a 2 x 2 system for V and U.  All parts are
+// linear in these coefficients: 200 FP64 operations a cell, where the matrix
+// took 450; its m and F cotangents, in 64-bit terms, are the more accurate.
 __device__ bool ls_adjoint(const Physics& ph, double tdt, double rho, double chi,
                            const double y[8], const double ybar[8], double yin[8],
                            double& chibar) {
-  const double cr = ph.c_over_chat, icc = ph.inv_cchat, ic2 = ph.inv_c2;
+  const double cr = ph.c_over_chat, icc = ph.inv_cchat, ic2 = ph.inv_c2, ic = ph.inv_c;
   const double irho = rcp_pos(rho);
-  const double Cv = rho * ph.cv_spec, iCv = rcp_pos(Cv);
+  const double iCv = irho * ph.inv_cv_spec;
   const bool o2 = ph.vc_order == 2;
   const double Eg = y[0], E = y[4];
-  const double m[3] = {y[1], y[2], y[3]}, F[3] = {y[5], y[6], y[7]};
-  double v[3], Ft[3];
+  double v[3], u[3];  // u: Ft
 #pragma unroll
   for (int i = 0; i < 3; ++i) {
-    v[i] = m[i] * irho;
-    Ft[i] = F[i] * ph.inv_c;
+    v[i] = y[1 + i] * irho;
+    u[i] = y[5 + i] * ic;
   }
-  const double Ek = 0.5 * (m[0] * v[0] + m[1] * v[1] + m[2] * v[2]);
-  const double T = (Eg - Ek) * iCv;
+  const double svv = dot3(v, v), svu = dot3(v, u), suu = dot3(u, u);
+  const double T = (Eg - 0.5 * rho * svv) * iCv;
   const double T3 = T * T * T;
   const double B = ph.a_rad * T3 * T, Bp = 4.0 * ph.a_rad * T3;
-  const double b2 = (v[0] * v[0] + v[1] * v[1] + v[2] * v[2]) * ic2;
-  const double g = o2 ? 1.0 + 0.5 * b2 : 1.0;
-  const double w = (v[0] * F[0] + v[1] * F[1] + v[2] * F[2]) * ic2;
+  const double g = o2 ? fma(0.5 * ic2, svv, 1.0) : 1.0;
   const double dk = ph.chat * tdt;  // dk/dchi
   const double k = dk * chi;
   // closure coefficients of P = ha I + hb Ft Ft^T and their partials
@@ -461,104 +422,69 @@ __device__ bool ls_adjoint(const Physics& ph, double tdt, double rho, double chi
     ha = E * (1.0 / 3.0);
     hb = 0.0;
     ha_E = 1.0 / 3.0;
+  } else if (lt_nn(E * E, suu)) {
+    const double iF2 = rcp_pos(suu);
+    ha = 0.0;
+    hb = E * iF2;
+    hb_E = iF2;
+    hb_F2 = -E * iF2 * iF2;
   } else {
-    double F2 = Ft[0] * Ft[0] + Ft[1] * Ft[1] + Ft[2] * Ft[2];
-    if (lt_nn(E * E, F2)) {
-      double iF2 = rcp_pos(F2);
-      ha = 0.0;
-      hb = E * iF2;
-      hb_E = iF2;
-      hb_F2 = -E * iF2 * iF2;
-    } else {
-      double x = 4.0 * E * E - 3.0 * F2;
-      double ir = rsqrt_pos(x), r = x * ir;
-      ha = (r - E) * (1.0 / 3.0);
-      hb = 3.0 * rcp_pos(2.0 * E + r);
-      double r_E = 4.0 * E * ir, r_F2 = -1.5 * ir;
-      ha_E = (r_E - 1.0) * (1.0 / 3.0);
-      ha_F2 = r_F2 * (1.0 / 3.0);
-      double hb2 = hb * hb * (1.0 / 3.0);
-      hb_E = -hb2 * (2.0 + r_E);
-      hb_F2 = -hb2 * r_F2;
-    }
+    const double x = fma(-0.75, suu, E * E);
+    const double ih = rsqrt_pos(x), h = x * ih;
+    const double w = rcp_pos(E + h), hb2 = 0.75 * w * w;
+    const double h2E = 2.0 * E * ih;
+    ha = fma(2.0, h, -E) * (1.0 / 3.0);
+    hb = 1.5 * w;
+    ha_E = (h2E - 1.0) * (1.0 / 3.0);
+    ha_F2 = -0.25 * ih;
+    hb_E = -hb2 * (2.0 + h2E);
+    hb_F2 = hb2 * 0.75 * ih;
   }
-  const double vFt = v[0] * Ft[0] + v[1] * Ft[1] + v[2] * Ft[2];
+  // R = k[(B - E) g + v.F/c^2]: dR/dEgas; dR/dm = mv v + mu Ft per unit of m;
+  // dR/dF with m = p - F/(c chat) folded in = ev v + eu Ft
+  const double kB = k * Bp * iCv, kr = k * irho, kc = k * ic, q = B - E;
+  const double R_Eg = g * kB;
+  const double mv = o2 ? fma(kr * ic2, q, -R_Eg) : -R_Eg, mu = kr * ic;
+  const double ev = fma(-icc, mv, k * ic2), eu = -icc * mu;
+  // flux rows: d/dEgas = -kB v, d/dE = bv v + bu Ft, d/dF = al I + vv v v + ..
+  const double Bh = B + ha, kg1 = fma(k, g, 1.0), kh = kr * hb;
+  const double bv = -k * ha_E, bu = -k * hb_E * svu;
+  const double o = o2 ? mu : 0.0;
+  const double al = fma(-kc * hb, svu, fma(icc * kr, Bh, kg1));
+  const double vv = -icc * kB, vu = -2.0 * kc * ha_F2, uv = -fma(kc, hb, icc * o);
+  const double uu = fma(-2.0 * kc * hb_F2, svu, icc * kh);
 
-  // R = k[(B - E) g + w] and its partials; m-partials are per unit of m
-  const double R_Eg = k * g * Bp * iCv;
-  const double R_E = -k * g;
-  double R_F[3], R_m[3];
+  const double x0 = ybar[0], x1 = ybar[4];
+  double x[3];
 #pragma unroll
-  for (int i = 0; i < 3; ++i) {
-    R_F[i] = k * v[i] * ic2;
-    R_m[i] = k * irho * (-g * Bp * v[i] * rho * iCv + (o2 ? (B - E) * v[i] * ic2 : 0.0) +
-                         F[i] * ic2);
-  }
-  const double R_chi = dk * ((B - E) * g + w);
+  for (int j = 0; j < 3; ++j) x[j] = fma(-icc, ybar[1 + j], ybar[5 + j]);
+  const double id = rcp_pos(fma(cr, R_Eg, kg1));
+  const double m0 = fma(-cr, x0, x1) * id, mV = -fma(cr, kB, bv) * id, mU = -bu * id;
+  const double AV = fma(-ev, mV, vv), AU = fma(-ev, mU, uv), A0 = -ev * m0;
+  const double BV = fma(-eu, mV, vu), BU = fma(-eu, mU, uu), B0 = -eu * m0;
+  const double M11 = fma(svv, AV, fma(svu, BV, al)), M12 = fma(svv, AU, svu * BU);
+  const double M21 = fma(svu, AV, suu * BV), M22 = fma(svu, AU, fma(suu, BU, al));
+  const double r1 = fma(-svv, A0, fma(-svu, B0, dot3(v, x)));
+  const double r2 = fma(-svu, A0, fma(-suu, B0, dot3(u, x)));
+  const double det = fma(M11, M22, -M12 * M21);
+  const long long db = dbits(det) & kMag, ab = dbits(al) & kMag;
+  if (db == 0 || db >= kInfBits || ab == 0 || ab >= kInfBits) return false;
+  const double idet = copysign(rcp_pos(fabs(det)), det);
+  const double V = fma(r1, M22, -M12 * r2) * idet, U = fma(M11, r2, -M21 * r1) * idet;
+  const double m1 = fma(mV, V, fma(mU, U, m0));
+  const double ca = fma(AV, V, fma(AU, U, A0)), cb = fma(BV, V, fma(BU, U, B0));
+  const double ial = copysign(rcp_pos(fabs(al)), al);
 
-  // Jacobian J[row][col]: rows (G, E, F1..3); cols (Egas, E, F1..3) with
-  // m = p - F/(c chat) folded in, then (p1..3), then chi.
-  double Jx[5][5], Jp[5][3], Jc[5];
-  Jx[0][0] = 1.0 + cr * R_Eg;
-  Jx[0][1] = cr * R_E;
-  Jx[1][0] = -R_Eg;
-  Jx[1][1] = 1.0 - R_E;
+  yin[0] = fma(R_Eg, m1, fma(kB, V, x0));
+  yin[4] = fma(cr, yin[0], m1);
+  chibar = dk * (fma(q, g, svu * ic) * m1 - fma(fma(ph.c, g, -hb * svu), U, -Bh * V));
+  const double Pv = fma(mv, m1, -fma(o, U, kB * V)), Pu = fma(mu, m1, kh * U), Pm = kr * Bh;
 #pragma unroll
   for (int j = 0; j < 3; ++j) {
-    double RFt = R_F[j] - R_m[j] * icc;
-    Jx[0][2 + j] = cr * RFt;
-    Jx[1][2 + j] = -RFt;
-    Jp[0][j] = cr * R_m[j];
-    Jp[1][j] = -R_m[j];
-  }
-  Jc[0] = cr * R_chi;
-  Jc[1] = -R_chi;
-  // r_F,i = F_i (1 + k g) - F_i(t) - k S_i,  S_i = B v_i + ha v_i + hb (v.Ft) Ft_i
-#pragma unroll
-  for (int i = 0; i < 3; ++i) {
-    double S_i = B * v[i] + ha * v[i] + hb * vFt * Ft[i];
-    Jx[2 + i][0] = -k * Bp * iCv * v[i];
-    Jx[2 + i][1] = -k * (ha_E * v[i] + hb_E * vFt * Ft[i]);
-    Jc[2 + i] = dk * (F[i] * g - S_i);
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-      double dij = i == j ? 1.0 : 0.0;
-      // partial in F_j at fixed m
-      double dS_F = ph.inv_c * (2.0 * Ft[j] * (ha_F2 * v[i] + hb_F2 * vFt * Ft[i]) +
-                                hb * v[j] * Ft[i] + hb * vFt * dij);
-      double pF = dij * (1.0 + k * g) - k * dS_F;
-      // partial in m_j
-      double dS_m = -Bp * iCv * v[i] * v[j] + (B * dij + ha * dij + hb * Ft[i] * Ft[j]) * irho;
-      double pm = F[i] * k * (o2 ? v[j] * irho * ic2 : 0.0) - k * dS_m;
-      Jx[2 + i][2 + j] = pF - pm * icc;
-      Jp[2 + i][j] = pm;
-    }
-  }
-  // (dr/dx)^T lambda = xbar,  xbar = (Egas, E, F - m/(c chat)) cotangents
-  double M[5][5], lam[5];
-#pragma unroll
-  for (int r = 0; r < 5; ++r)
-#pragma unroll
-    for (int s = 0; s < 5; ++s) M[r][s] = Jx[s][r];
-  lam[0] = ybar[0];
-  lam[1] = ybar[4];
-#pragma unroll
-  for (int j = 0; j < 3; ++j) lam[2 + j] = ybar[5 + j] - ybar[1 + j] * icc;
-  if (!solve5(M, lam)) return false;
-  yin[0] = lam[0];
-  yin[4] = lam[1];
-  double cs = 0.0;
-#pragma unroll
-  for (int r = 0; r < 5; ++r) cs += Jc[r] * lam[r];
-  chibar = -cs;
-#pragma unroll
-  for (int j = 0; j < 3; ++j) {
-    double s = 0.0;
-#pragma unroll
-    for (int r = 0; r < 5; ++r) s += Jp[r][j] * lam[r];
-    double pbar = ybar[1 + j] - s;
+    const double l = fma(-v[j], ca, fma(-u[j], cb, x[j])) * ial;
+    const double pbar = fma(Pv, v[j], fma(Pu, u[j], fma(Pm, l, ybar[1 + j])));
     yin[1 + j] = pbar;
-    yin[5 + j] = lam[2 + j] + pbar * icc;
+    yin[5 + j] = fma(pbar, icc, l);
   }
   return true;
 }
@@ -674,7 +600,11 @@ static void face_layout(const Geometry& g, long long off[3], long long nface[3])
 cudaError_t launch_adjoint_step(const AdjointStep& S, cudaStream_t s) {
   const Geometry& g = S.g;
   const int N = g.ncell;
-  const int nb = (N + 255) / 256;
+  // one thread a cell or face: blocks of 64 spread a small grid over the SMs
+  // (16 SMs' FP64 pipes did the work of a 64^2 grid in blocks of 256), blocks
+  // of 256 where there are enough of them
+  const int bs = N < 152 * 256 * 2 ? 64 : 256;
+  const int nb = (N + bs - 1) / bs;
   CellArgs C;
   C.g = g;
   C.ph = S.ph;
@@ -698,29 +628,30 @@ cudaError_t launch_adjoint_step(const AdjointStep& S, cudaStream_t s) {
   face_layout(g, F.off, F.nface);
   F.total = 0;
   for (int d = 0; d < g.ndim; ++d) F.total += F.nface[d];
-  const int fb = (int)((F.total + 255) / 256);
+  const int fb = (int)((F.total + bs - 1) / bs);
+  for (int d = 0; d < 3; ++d) F.eps[d] = S.eps[d];
 
   // A: stage-2 local solve at y1
   C.tdt = 0.5 * S.dt;
   for (int q = 0; q < NY; ++q) C.ys[q] = S.y1 + (size_t)q * N;
   C.fp = S.pending_fp ? S.fp : nullptr;
-  cell_adj_kernel<0><<<nb, 256, 0, s>>>(C);
+  cell_adj_kernel<0><<<nb, bs, 0, s>>>(C);
   // B: transport at yh, weight dt/2, cotangent q
   for (int q = 0; q < 4; ++q) {
     F.y[q] = S.yh + (size_t)(Y_ERAD + q) * N;
     F.cot[q] = S.q + (size_t)(Y_ERAD + q) * N;
   }
-  F.alpha = 0.5 * S.dt;
-  face_vjp_kernel<<<fb, 256, 0, s>>>(F);
+  flux_weights(g, S.ph, false, 0.5 * S.dt, F.wE, F.wF);
+  face_vjp_kernel<<<fb, bs, 0, s>>>(F);
   // C: stage-1 local solve at yh
   C.tdt = S.dt;
   for (int q = 0; q < NY; ++q) C.ys[q] = S.yh + (size_t)q * N;
   C.fp = S.fp;
-  cell_adj_kernel<1><<<nb, 256, 0, s>>>(C);
+  cell_adj_kernel<1><<<nb, bs, 0, s>>>(C);
   // D: transport at y(n), weight dt, cotangent q'
   for (int q = 0; q < 4; ++q) F.y[q] = S.yn + (size_t)(Y_ERAD + q) * N;
-  F.alpha = S.dt;
-  face_vjp_kernel<<<fb, 256, 0, s>>>(F);
+  flux_weights(g, S.ph, false, S.dt, F.wE, F.wF);
+  face_vjp_kernel<<<fb, bs, 0, s>>>(F);
   return cudaGetLastError();
 }
 

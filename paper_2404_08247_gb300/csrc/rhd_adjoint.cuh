@@ -16,6 +16,7 @@ struct AdjointStep {
   int step;                 // step index (for the status block)
   const double* rho;
   const double* kappa;
+  const double* eps[3];     // TAU mode: factors of the +d faces (launch_tau_eps)
   const double* yn;         // tape: y(n), y(n+1/2), y(n+1), slot-major NY * ncell each
   const double* yh;
   const double* y1;

@@ -1266,7 +1266,13 @@ rhd_status rhd_adjoint(rhd_ctx* c, const double* tape, int64_t count, int nsteps
     }
   }
   CUDA_TRY(c, launch_status_reset(c->d_status, c->stream));
+  if (c->p.hll_mode == RHD_HLL_TAU && c->eps_dirty) {
+    CUDA_TRY(c, launch_tau_eps(c->g, c->rho, c->kappa, c->ph.kappa_F_ratio, c->eps, c->stream));
+    c->launches += 1;
+    c->eps_dirty = false;
+  }
   AdjointStep A;
+  for (int d = 0; d < 3; ++d) A.eps[d] = c->eps[d];
   A.g = c->g;
   A.ph = c->ph;
   A.dt = dt;
