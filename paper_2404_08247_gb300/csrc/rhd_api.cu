@@ -328,6 +328,8 @@ void rhd::fill_geometry(const rhd_params* p, Geometry& g, Physics& ph) {
   ph.scheme = p->scheme;
   ph.kappa_T_exp = p->kappa_T_exp;
   ph.inv_kappa_T_ref = 1.0 / p->kappa_T_ref;
+  if (std::fabs(p->kappa_T_exp) <= 8.0 && p->kappa_T_exp == std::floor(p->kappa_T_exp))
+    ph.kappa_T_int = (int)p->kappa_T_exp;
   ph.kappa_P_ratio = p->kappa_P_ratio;
   ph.kappa_F_ratio = p->kappa_F_ratio;
   ph.reconstruction = p->reconstruction;

@@ -81,6 +81,7 @@ struct Physics {
   int scheme;              // rhd_scheme
   double kappa_T_exp;      // chi = kappa rho (T / T_ref)^kappa_T_exp
   double inv_kappa_T_ref;  // 1 / T_ref
+  int kappa_T_int;         // kappa_T_exp where it is a whole number up to 8, else 0
   double kappa_P_ratio;    // chi_0P / chi_0E
   double kappa_F_ratio;    // chi_0F / chi_0E
   int reconstruction;      // rhd_recon
@@ -634,6 +635,25 @@ __device__ __forceinline__ bool quartic_start(double a4, double rhs, double T0, 
 // to rounding.
 // GEN: compiled with the temperature-dependent opacity; the default physics
 // (constant chi) uses the GEN = false copy, free of that branch.
+// (T/T_ref)^p of chi = kappa rho (T/T_ref)^p.  Whole exponents (the Marshak
+// wave's -3) by a product that carries its rounding errors (fused
+// multiply-adds; Dekker 1971) and one reciprocal: within 1 ulp, and 13 FP64
+// operations for -3, where pow takes several times that in every Newton update.
+__device__ __forceinline__ double opacity_power(const Physics& ph, double x) {
+  const int n = ph.kappa_T_int < 0 ? -ph.kappa_T_int : ph.kappa_T_int;
+  if (n == 0) return pow(x, ph.kappa_T_exp);
+  double hi = x, lo = 0.0;
+  for (int i = 1; i < n; ++i) {
+    const double p = mul(hi, x);
+    lo = fma(lo, x, fma(hi, x, -p));
+    hi = p;
+  }
+  if (!seed_range(hi)) return pow(x, ph.kappa_T_exp);
+  if (ph.kappa_T_int > 0) return add(hi, lo);
+  const double r = rcp_pos(hi);
+  return fma(mul(-lo, r), r, r);
+}
+
 constexpr double kNear = 1e4;  // in units of the Newton tolerance
 
 template <bool MIXED, bool GEN>
@@ -731,7 +751,7 @@ __device__ __forceinline__ int local_solve(const Physics& ph, double tdt, double
           break;
         }
         if (vary) {
-          k = mul(k0, pow(mul(T, ph.inv_kappa_T_ref), ph.kappa_T_exp));
+          k = mul(k0, opacity_power(ph, mul(T, ph.inv_kappa_T_ref)));
           kg = fma(k, h, k);
           kw = mul(k, w);
         }
@@ -887,7 +907,7 @@ __device__ int local_solve_nongrey(const Physics& ph, double tdt, double rho, do
   double vDv = vdv_of(v);
   double kE = k0, kP = rP * k0, kF = rF * k0;
   auto set_k = [&](double T) {
-    kE = vary ? k0 * pow(T * ph.inv_kappa_T_ref, ph.kappa_T_exp) : k0;
+    kE = vary ? k0 * opacity_power(ph, mul(T, ph.inv_kappa_T_ref)) : k0;
     kP = rP * kE;
     kF = rF * kE;
   };
