@@ -191,23 +191,34 @@ __device__ __forceinline__ double dot3(const double a[3], const double b[3]) {
   return fma(a[2], b[2], fma(a[1], b[1], mul(a[0], b[0])));
 }
 
-// x/2, and the magnitude bits of x/4, exactly: the exponent field lowered on
-// the integer pipe (outside the normal range: the product)
+// x/2, and the magnitude bits of x/4: the exponent field lowered on the integer
+// pipe; exact, but zero below 2^-1021 and 2^-1020.  (A product for that range
+// would issue, predicated off, with every use: 32 slots of the FP64 pipe a
+// cell.)
 __device__ __forceinline__ double half_of(double x) {
-  const int e = (int)((dbits(x) >> 52) & 0x7ff);
-  return e > 1 && e < 0x7ff ? __longlong_as_double(dbits(x) - (1ll << 52)) : 0.5 * x;
+  const long long b = dbits(x), a = b & kMag;
+  const long long h = a >= kInfBits ? a : a >= (2ll << 52) ? a - (1ll << 52) : 0ll;
+  return __longlong_as_double(h | (b & ~kMag));
 }
 __device__ __forceinline__ long long quarter_bits(double x) {
   const long long a = abs_bits(x);
-  return a >= (3ll << 52) && a < kInfBits ? a - (2ll << 52) : abs_bits(0.25 * x);
+  return a >= kInfBits ? a : a >= (3ll << 52) ? a - (2ll << 52) : 0ll;
 }
-// a float as a double, exactly, by integer operations (the conversion where it
-// is zero, subnormal or not finite)
+// a float as a double, exactly, by integer operations
 __device__ __forceinline__ double widen(float f) {
-  const unsigned u = __float_as_uint(f), e = (u >> 23) & 0xffu;
-  if (e == 0u || e == 0xffu) return (double)f;
-  const long long m = ((long long)(u & 0x7fffffffu) << 29) + (896ll << 52);
-  return __longlong_as_double(m | ((long long)(u & 0x80000000u) << 32));
+  const unsigned u = __float_as_uint(f), a = u & 0x7fffffffu;
+  unsigned m = a, e = 896u;  // the magnitude bits, the exponent's offset
+  if (a >= 0x7f800000u) {
+    e = 0x7ffu - 0xffu;  // infinity, NaN
+  } else if (a < 0x00800000u) {
+    // subnormal: the leading bit to the implicit place, the exponent from its
+    // position; zero stays zero
+    const int sh = __clz((int)a) - 8;
+    m = a == 0u ? 0u : (a << sh) & 0x007fffffu;
+    e = a == 0u ? 0u : 897u - (unsigned)sh;
+  }
+  const long long d = ((long long)m << 29) + ((long long)e << 52);
+  return __longlong_as_double(d | ((long long)(u & 0x80000000u) << 32));
 }
 
 // 1/x to about 2^-21 for x > 0, off the FP64 pipe (outside the single-precision
@@ -308,8 +319,9 @@ __device__ __forceinline__ double ppm_edge_d(double u0, double l, double r) {
   const long long ba = dbits(a), bb = dbits(b);
   const long long ma = ba & kMag, mb = bb & kMag;
   const bool mono = ((ba ^ bb) >= 0) & (ma != 0) & (mb != 0);
-  const bool plain = mb >= (1ll << 52) && mb < kInfBits - (1ll << 52);
-  const long long m = min(ma, plain ? mb + (1ll << 52) : abs_bits(b + b));
+  // (2|b| of a subnormal b doubles its bits; none is below infinity above)
+  const long long b2 = mb < (1ll << 52) ? 2 * mb : min(mb + (1ll << 52), kInfBits);
+  const long long m = min(ma, b2);
   const double s = __longlong_as_double(mono ? (m | (ba & ~kMag)) : 0ll);
   return LEFT ? u0 - s : u0 + s;
 }
@@ -445,20 +457,31 @@ __device__ __forceinline__ void m1_coeffs(double E, const double Ft[3], double& 
 // (2h - E)/3 I + 3/2/(E + h) Ft Ft^T; E^2 and |Ft|^2 serve the limit as well
 // (a flux scaled back has |Ft| = E, so P = E n n).
 __device__ __forceinline__ void face_side(int d, double q[4], int closure, double P[3]) {
-  const double E = q[0], E2 = mul(E, E);
-  double F2 = dot3(q + 1, q + 1);
-  if (lt_nn(E2, F2)) {
-    const double sc = mul(E, rsqrt_pos(F2));
+  const double E = q[0], E2 = mul(E, E), F2 = dot3(q + 1, q + 1);
+  const bool over = lt_nn(E2, F2);
+  // one root serves both: h, and above the limit 1/|Ft|
+  const double x = over ? F2 : fma(-0.75, F2, E2);
+  double y, h, corr = 0.0;
+  if (seed_range(x)) {
+    double t;
+    y = seed_double(rsqrtf(seed_float(x)));
+    corr = rsqrt_corr(x, y, t);
+    h = fma(t, corr, t);
+  } else {
+    h = sqrt(x);
+    y = 1.0 / h;
+  }
+  if (over) {
+    const double sc = mul(E, fma(y, corr, y));
 #pragma unroll
     for (int j = 0; j < 3; ++j) q[1 + j] = mul(q[1 + j], sc);
-    F2 = E2;
+    h = half_of(E);
   }
   if (closure == RHD_CLOSURE_EDDINGTON) {
     P[0] = P[1] = P[2] = 0.0;
     P[d] = mul(E, 1.0 / 3.0);
     return;
   }
-  const double h = sqrt_pos(fma(-0.75, F2, E2));
   const double ha = mul(fma(2.0, h, -E), 1.0 / 3.0);
   const double t = mul(mul(1.5, rcp_pos(add(E, h))), q[1 + d]);
 #pragma unroll

@@ -189,11 +189,18 @@ __device__ __forceinline__ double face_eps(const StageArgs& A, int d, int cx, in
 
 // Mixed precision: x as a pair of floats with hi + lo = x to 2^-47 |x|.  hi
 // is x with its mantissa cut to 24 bits, lo the rest rounded to float, both by
-// integer operations within the float exponent range.  A
+// integer operations within the float exponent range (and zero; the rest is a
+// call, whose conversions would else issue with every value).  A
 // difference of two neighbours, (b_hi - a_hi) + (b_lo - a_lo), is then good
 // to single precision of the difference itself, where the difference of the
 // rounded values would carry an error of an ulp of the values: the MC slopes
 // and face states of the mixed transport are formed that way.
+__device__ __noinline__ float split_rest(double x, float* lo) {
+  const float hi = (float)x;
+  *lo = (float)(x - (double)hi);
+  return hi;
+}
+
 __device__ __forceinline__ void split_hilo(double x, float& hi, float& lo) {
   const long long b = __double_as_longlong(x);
   const int e = (int)((b >> 52) & 0x7ff);
@@ -203,9 +210,13 @@ __device__ __forceinline__ void split_hilo(double x, float& hi, float& lo) {
     // the low 29 bits, in units of 2^(e - 1023 - 52)
     lo = (float)(unsigned)(b & 0x1fffffffll) *
          __uint_as_float(sign | ((unsigned)(e - 896 - 52) << 23));
+  } else if ((b & 0x7fffffffffffffffll) == 0) {
+    hi = __int_as_float((int)(b >> 32));
+    lo = 0.f;
   } else {
-    hi = (float)x;
-    lo = (float)(x - (double)hi);
+    float l;
+    hi = split_rest(x, &l);
+    lo = l;
   }
 }
 
