@@ -195,7 +195,7 @@ __device__ __forceinline__ double face_eps(const StageArgs& A, int d, int cx, in
 // to single precision of the difference itself, where the difference of the
 // rounded values would carry an error of an ulp of the values: the MC slopes
 // and face states of the mixed transport are formed that way.
-__device__ __noinline__ float split_rest(double x, float* lo) {
+static __device__ __noinline__ float split_rest(double x, float* lo) {
   const float hi = (float)x;
   *lo = (float)(x - (double)hi);
   return hi;
