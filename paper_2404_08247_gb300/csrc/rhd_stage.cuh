@@ -33,14 +33,17 @@ __global__ void __launch_bounds__(TileOf<NDIM, PPM, SMALL>::NT,
 }
 
 // The tile and the planes per block of a stage over a grid (launches over parts
-// of it, which run side by side, take the whole grid's).  Both candidates (the large tile; the small one, whose
-// faces take more warp rounds a cell) and 1 to 16 planes a block (a block adds
-// a z face a column and its ghost planes' loads) are priced, and the cheapest
-// is taken.  Prices are FP64 instructions a warp, of which an SM's pipe issues
-// one in 16 cycles: a face, a z face and a cell's slopes, update and solve.  A
-// launch takes the longer of its busiest SM's instructions and of one block's
-// own chain (about 28 cycles an instruction and 6000 a plane for the pair
-// arithmetic and barriers) for each round of resident blocks.
+// of it, which run side by side, take the whole grid's).  Both candidates
+// (the large tile; the small one, whose faces take more warp rounds a cell)
+// and 1 to 16 planes a block (a block adds a z face a column and its ghost
+// planes' loads) are priced, and the cheapest is taken.  Prices are FP64
+// instructions a warp: a face, a z face and a cell's slopes, update and solve.
+// The busiest SM issues its instructions at one in 16 cycles, slowed by (1 + 6/w)
+// when w warps are resident: 73 % of the pipe with 16 warps, 50 to 57 % with
+// 8, 11 to 14 % with one, as measured.  Against the large tile with 8 planes a
+// block everywhere: a 40 x 37 x 33 box, five steps, 5.3 -> 2.2 ms; a 256-cell
+// row, 50 steps, 4.6 -> 3.5 ms; 256^3, where both price 8 or 16 planes alike,
+// unchanged.
 struct TilePlan {
   bool small;
   int lz;
@@ -65,12 +68,9 @@ inline TilePlan plan_tiles(const Geometry& g, bool mixed, bool ppm, bool allow_s
       if (nb[1] > 65535 || nb[2] > 65535) continue;
       const double z = g.ndim == 3 ? face : 0.0;
       const double plane = face * (rx + ry) + (cell + z) * nw, start = 2.0 * z * nw;
-      const double chain = face * ((rx + nw - 1) / nw + (ry + nw - 1) / nw) + cell + z;
       const long long per_sm = (nb[0] * nb[1] * nb[2] + kSMs - 1) / kSMs;
-      const double busy = 16.0 * per_sm * (lz * plane + start);
-      const double wait = (double)((per_sm + resident - 1) / resident) *
-                          (lz * (28.0 * chain + 6000.0) + 28.0 * 2.0 * z);
-      const double t = busy > wait ? busy : wait;
+      const double warps = nw * (double)(per_sm < resident ? per_sm : resident);
+      const double t = per_sm * (lz * plane + start) * (1.0 + 6.0 / warps);
       if (tbest == 0.0 || t < tbest) {
         tbest = t;
         best.small = small != 0;

@@ -83,7 +83,9 @@ struct SmemT {
   // the same place: the faces -1 .. TX + 1 of the tile's rows, so that each is
   // computed once and not for the three faces that read it.  They share the
   // Colella-Sekora march's second differences' place (which recomputes its
-  // interface values): with that, two blocks of the 3-D tile fit an SM.
+  // interface values): with that, two blocks of the 3-D tile fit an SM.  A
+  // face's states take 56 FP64 operations instead of 132: a 128 x 96 x 110 box,
+  // three steps, 20.5 ms instead of 24.0.
   static constexpr bool IFACE = T::PPM && sizeof(R) == sizeof(double);
   static constexpr int AX = IFACE ? T::TY * (T::TX + 3) : 0;  // per field
   static constexpr int AY = IFACE && T::NDIM >= 2 ? (T::TY + 3) * T::TX : 0;
@@ -99,7 +101,8 @@ struct SmemT {
   static constexpr size_t ISO_OFF = sizeof(R) * (RING + FX + FY + CZ);
   // FP64 PLM: half slopes along x of the tile's cells and one beyond on each
   // side, and along y, so that each is computed once and not for both faces
-  // of its cell
+  // of its cell (bound by the FP64 pipe: with the shared closure terms of
+  // face_side two steps of a 256^3 box take 97.7 ms instead of 112.0)
   static constexpr bool SLOPES = !T::PPM && sizeof(R) == sizeof(double);
   static constexpr int SX = SLOPES ? T::TY * (T::TX + 2) : 0;            // per field
   static constexpr int SY = SLOPES && T::NDIM >= 2 ? (T::TY + 2) * T::TX : 0;
