@@ -156,6 +156,8 @@ typedef struct {
   int64_t fail_cell;   /* smallest failing cell index, -1 if none */
   int fail_step;       /* step (within the call) that failed, -1 if none */
   int fail_stage;      /* 1 or 2, 0 if none */
+  /* the iteration counts are those of the whole iteration, whichever
+   * arithmetic (pairs of floats or double) a pass ran in */
   int max_newton;      /* most Newton updates of any local solve */
   int max_outer;       /* most outer passes of any local solve */
   int64_t sum_newton;  /* total Newton updates */
