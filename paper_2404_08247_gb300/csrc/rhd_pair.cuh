@@ -5,10 +5,12 @@
 // product uses the fused multiply-add (Dekker 1971; Knuth, The Art of
 // Computer Programming, vol. 2, Sec. 4.2.2; Hida, Li & Bailey 2001).  The
 // single-precision pipe of this GPU has 64 times the throughput of the
-// double-precision one, so an operation on pairs (7 to 11 instructions) costs
-// a fraction of a double-precision one's pipe time.  Results are good to a few
+// double-precision one, so an operation on pairs (4 to 11 instructions) costs
+// a fraction of a double-precision one's pipe time.  Sums are renormalised (a
+// cancellation may leave everything in lo); products, reciprocals and roots
+// are not, their lo being a few ulps of hi at most.  Results are good to a few
 // 2^-47 of the operands: enough to bring an iteration next to its fixed point,
-// which double-precision passes then settle.
+// which a double-precision pass then settles.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -36,7 +38,11 @@ __device__ __forceinline__ Pair operator-(Pair a, Pair b) { return a + (-b); }
 __device__ __forceinline__ Pair operator*(Pair a, Pair b) {
   const float p = __fmul_rn(a.hi, b.hi);
   const float e = __fmaf_rn(a.lo, b.hi, __fmaf_rn(a.hi, b.lo, __fmaf_rn(a.hi, b.hi, -p)));
-  return pair_norm(p, e);
+  return {p, e};
+}
+__device__ __forceinline__ Pair operator*(Pair a, float b) {
+  const float p = __fmul_rn(a.hi, b);
+  return {p, __fmaf_rn(a.lo, b, __fmaf_rn(a.hi, b, -p))};
 }
 // product with a power of two (exact)
 __device__ __forceinline__ Pair scaled(Pair a, float s) { return {a.hi * s, a.lo * s}; }
@@ -51,14 +57,14 @@ __device__ __forceinline__ Pair operator+(Pair a, float b) {
 __device__ __forceinline__ Pair recip(Pair a) {
   const float r = __fdividef(1.f, a.hi);
   const float e = __fmaf_rn(-a.lo, r, __fmaf_rn(-a.hi, r, 1.f));
-  return pair_norm(r, __fmul_rn(r, __fmaf_rn(e, e, e)));
+  return {r, __fmul_rn(r, __fmaf_rn(e, e, e))};
 }
 // sqrt(a), a > 0: s = a rsqrt(a) and one Newton correction
 __device__ __forceinline__ Pair root(Pair a) {
   const float y = rsqrtf(a.hi);
   const float s = __fmul_rn(a.hi, y);
   const float t = __fadd_rn(__fmaf_rn(-s, s, a.hi), a.lo);
-  return pair_norm(s, __fmul_rn(t, 0.5f * y));
+  return {s, __fmul_rn(t, 0.5f * y)};
 }
 __device__ __forceinline__ Pair square(Pair a) { return a * a; }
 __device__ __forceinline__ float value(Pair a) { return a.hi; }
