@@ -81,7 +81,7 @@ __global__ void __launch_bounds__(kBatchThreads, 2) batch_kernel(const BatchArgs
     const ProblemDesc& P = B.probs[w.prob];
     // the item's arguments in shared memory, where the tile reads them as the
     // grid kernels read their launch arguments: held in registers they cost
-    // 700 bytes of spills a thread
+    // 700 bytes of spills a thread (now 196, the solve being a call)
     if (threadIdx.x == 0) {
       A.g = P.g;
       A.ph = P.ph;
