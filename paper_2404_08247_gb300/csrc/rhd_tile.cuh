@@ -494,6 +494,7 @@ __device__ __forceinline__ void stage_tile(const StageArgs& A, int x0, int y0, i
   constexpr int NDIM = T::NDIM;
   constexpr int TX = T::TX, TY = T::TY, NT = TX * TY;
   constexpr bool MIXED = sizeof(R) == sizeof(float);
+  constexpr bool EARLY = NDIM == 3 && S::SLOPES;  // the next plane is loaded before its turn
   R* ring = reinterpret_cast<R*>(smem_raw);
   R* fxs = ring + S::RING;
   R* fys = fxs + S::FX;
@@ -609,17 +610,32 @@ __device__ __forceinline__ void stage_tile(const StageArgs& A, int x0, int y0, i
     }
     R eps = (R)face_eps(A, 2, cx, cy, kbeg - 1);
     zbad = !face_hll<R>(2, L, Rr, eps, chat, ph.closure, zlo, zlo_iso);
-    __syncthreads();  // plane kbeg-2's slot is reloaded by the first iteration
+    __syncthreads();  // every thread has read plane kbeg-2
+    if (EARLY) {
+      load_plane<T, R, GEN>(A, ring, (kbeg + 2) & 3, kbeg + 2, x0, y0);
+      __syncthreads();
+    }
   }
 
+  // Two barriers a plane (PPM in FP64: and its interface values').  The one
+  // after the faces, which the update reads: behind it the ring's plane k and the
+  // slopes are free, so none closes the loop, and a warp that has solved its cells
+  // goes on to the next plane while others solve.  And one before the x-faces,
+  // whose fluxes the update of plane k-1 has read then: in FP64 PLM behind the
+  // slopes, with the plane for the next iteration loaded before them (256^3, two
+  // steps: 85.6 ms instead of 87.8 with barriers at the load and the loop's end);
+  // else on top, behind the load (mixed precision with the FP64 order: 41.8 ms
+  // instead of 40.8 for four steps of 250 x 200 x 130).
   for (int k = kbeg; k < kend; ++k) {
-    if (NDIM == 3) {
-      constexpr int AHEAD = T::PPM ? 3 : 2;
-      load_plane<T, R, GEN>(A, ring, ring_slot<T>(k + AHEAD), k + AHEAD, x0, y0);
+    if constexpr (EARLY) {
+      // the slot of plane k-1, read for the last time by that plane's faces
+      if (k + 1 < kend) load_plane<T, R, GEN>(A, ring, (k + 3) & 3, k + 3, x0, y0);
     } else {
-      load_plane<T, R, GEN>(A, ring, 0, 0, x0, y0);
+      constexpr int AHEAD = T::PPM ? 3 : 2;
+      const int kl = NDIM == 3 ? k + AHEAD : 0;
+      load_plane<T, R, GEN>(A, ring, NDIM == 3 ? ring_slot<T>(kl) : 0, kl, x0, y0);
+      __syncthreads();
     }
-    __syncthreads();
     const R* pl = ring + (NDIM == 3 ? ring_slot<T>(k) : 0) * S::PLANE;
     bool bad = zbad;
 
@@ -696,7 +712,8 @@ __device__ __forceinline__ void stage_tile(const StageArgs& A, int x0, int y0, i
     }
 
     // ---- FP64 PLM: half slopes of plane k, each thread its own cell's, then
-    // those of the cells next to the tile
+    // those of the cells next to the tile (the last threads, which have one
+    // cell less to load)
     if constexpr (S::SLOPES) {
       auto slope = [&](int c, int st, double* out, int sn) {
         double um[4], u0[4], up[4];
@@ -709,7 +726,7 @@ __device__ __forceinline__ void stage_tile(const StageArgs& A, int x0, int y0, i
       slope(own, 1, sx + ty * (TX + 2) + tx + 1, S::SX);
       if (NDIM >= 2) slope(own, S::PW, sy + (ty + 1) * TX + tx, S::SY);
       constexpr int NY2 = NDIM >= 2 ? 2 * TX : 0;
-      for (int i = threadIdx.x; i < NY2 + 2 * TY; i += NT) {
+      for (int i = NT - 1 - threadIdx.x; i < NY2 + 2 * TY; i += NT) {
         if (NDIM >= 2 && i < NY2) {  // rows -1 and TY
           const int r = i < TX ? -1 : TY, x = i < TX ? i : i - TX;
           slope(x + T::HX + (r + T::HY) * S::PW, S::PW, sy + (r + 1) * TX + x, S::SY);
@@ -763,7 +780,8 @@ __device__ __forceinline__ void stage_tile(const StageArgs& A, int x0, int y0, i
       for (int q = 0; q < 4; ++q) fxs[q * TY * (TX + 1) + f] = out[q];
       if constexpr (MIXED) fxi[f] = iso;
     }
-    // ---- y-faces of plane k: face f lies between rows fj-1 and fj
+    // ---- y-faces of plane k: face f lies between rows fj-1 and fj (the first
+    // warp has the x-faces beyond NT, the last one the y-faces beyond NT)
     if (NDIM >= 2) {
       if (S::IFACE && !cs) {
         __syncthreads();  // every x-face has read its interface values
@@ -773,7 +791,7 @@ __device__ __forceinline__ void stage_tile(const StageArgs& A, int x0, int y0, i
         }
         __syncthreads();
       }
-      for (int f = threadIdx.x; f < TX * (TY + 1); f += NT) {
+      for (int f = (threadIdx.x + 32) % NT; f < TX * (TY + 1); f += NT) {
         int fi = f % TX, fj = f / TX;
         int c = fi + T::HX + (fj + T::HY) * S::PW;
         int xr = x0 + fi, yl = y0 + fj - 1;
@@ -896,9 +914,7 @@ __device__ __forceinline__ void stage_tile(const StageArgs& A, int x0, int y0, i
       }
       zlo_iso = zhi_iso;
     }
-    __syncthreads();
   }
-
 }
 
 // Block reduction of TileStats (warp shuffles, then one atomic per block).
