@@ -60,6 +60,15 @@ using Tile1P = TileT<1, 256, 1, true>;
 using Tile2P = TileT<2, 32, 8, true>;
 constexpr int kBatchThreads = 256;
 
+// dst = src by the block's threads, a word each
+template <class T>
+__device__ __forceinline__ void copy_words(T& dst, const T& src) {
+  static_assert(sizeof(T) % 4 == 0, "whole words");
+  int* d = reinterpret_cast<int*>(&dst);
+  const int* s = reinterpret_cast<const int*>(&src);
+  for (int i = threadIdx.x; i < (int)(sizeof(T) / 4); i += kBatchThreads) d[i] = __ldg(s + i);
+}
+
 // PPMX: the batch holds PPM problems (the kernel then carries both tile kinds)
 template <int STAGE, class T2, typename R, bool GEN, bool PPMX>
 __global__ void __launch_bounds__(kBatchThreads, 2) batch_kernel(const BatchArgs B) {
@@ -71,20 +80,25 @@ __global__ void __launch_bounds__(kBatchThreads, 2) batch_kernel(const BatchArgs
   __syncthreads();
   if (s_skip) return;  // a previous launch of this batch failed
   TileStats ts;
+  // Thread 0's: the next item, taken while the current one runs, so that the
+  // counter's latency is not waited for.  With an item's grid and physics copied
+  // by all threads 512 problems, mixed, take 225 ms for 500 steps instead of 233.
+  int next = 0;
+  if (threadIdx.x == 0) next = atomicAdd(B.counter, 1);
   for (;;) {
-    if (threadIdx.x == 0) s_item = atomicAdd(B.counter, 1);
-    __syncthreads();
+    if (threadIdx.x == 0) s_item = next;
+    __syncthreads();  // (every thread has left the last item's tile)
     const int it = s_item;
-    __syncthreads();  // every thread has read s_item before it is reused
     if (it >= B.nitems) break;
     const WorkItem w = B.items[it];
     const ProblemDesc& P = B.probs[w.prob];
     // the item's arguments in shared memory, where the tile reads them as the
     // grid kernels read their launch arguments: held in registers they cost
     // 700 bytes of spills a thread (now 196, the solve being a call)
+    copy_words(A.g, P.g);
+    copy_words(A.ph, P.ph);
     if (threadIdx.x == 0) {
-      A.g = P.g;
-      A.ph = P.ph;
+      next = atomicAdd(B.counter, 1);
       A.dt = P.dt;
       A.step = B.step;
       A.st = B.st;
