@@ -115,10 +115,19 @@ struct StageArgs {
   // factors of the low slab face (n0 n1)
   const double* halo[2] = {nullptr, nullptr};
   const double* eps_zlo = nullptr;
-  // the first cell of the launch along the slowest axis (z in 3-D, y in 2-D, x
-  // in 1-D) and the planes a 3-D block marches through
-  int lo = 0, lz = 1;
+  // the cells [lo, hi) of the launch along the slowest axis (z in 3-D, y in 2-D,
+  // x in 1-D) and the planes a 3-D block marches through, its last one fewer
+  int lo = 0, hi = 0, lz = 1;
 };
+
+// The planes [k0, k1) of block b of a 3-D launch over the planes [lo, hi): the
+// last block stops at the launch's end.  Launches over parts of one grid run
+// side by side (rhd_step_host), and the planes beyond belong to another one,
+// whose inputs this one has not waited for.
+__host__ __device__ inline void block_planes(int b, int lo, int hi, int lz, int& k0, int& k1) {
+  k0 = lo + b * lz;
+  k1 = k0 + lz < hi ? k0 + lz : hi;
+}
 
 // ghost planes a HALO face holds (the widest face stencil: PPM's 3)
 constexpr int HALO_PLANES = 3;

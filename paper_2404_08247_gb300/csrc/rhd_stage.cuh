@@ -26,14 +26,15 @@ __global__ void __launch_bounds__(TileOf<NDIM, PPM, SMALL>::NT,
   TileStats ts;
   const int x0 = blockIdx.x * T::TX + (NDIM == 1 ? A.lo : 0);
   const int y0 = blockIdx.y * T::TY + (NDIM == 2 ? A.lo : 0);
-  const int k0 = NDIM == 3 ? blockIdx.z * A.lz + A.lo : 0;
-  stage_tile<STAGE, T, R, GEN>(A, x0, y0, k0, NDIM == 3 ? min(k0 + A.lz, A.g.n[2]) : 1, smem_raw,
-                               ts);
+  int k0 = 0, k1 = 1;
+  if (NDIM == 3) block_planes(blockIdx.z, A.lo, A.hi, A.lz, k0, k1);
+  stage_tile<STAGE, T, R, GEN>(A, x0, y0, k0, k1, smem_raw, ts);
   flush_stats<T::NT>(A.st, ts);
 }
 
 // The tile and the planes per block of a stage over a grid (launches over parts
-// of it, which run side by side, take the whole grid's).  Both candidates
+// of it, which run side by side, take the whole grid's, and where a part's 8-plane
+// rows are an odd number its last blocks march 8 planes of 16).  Both candidates
 // (the large tile; the small one, whose faces take more warp rounds a cell)
 // and 1 to 16 planes a block (a block adds a z face a column and its ghost
 // planes' loads) are priced, and the cheapest is taken.  Prices are FP64
@@ -82,7 +83,7 @@ inline TilePlan plan_tiles(const Geometry& g, bool mixed, bool ppm, bool allow_s
 }
 
 template <int STAGE, int NDIM, typename R, bool GEN, bool PPM, bool SMALL>
-static cudaError_t launch_tile(const StageArgs& A, cudaStream_t s, int hi) {
+static cudaError_t launch_tile(const StageArgs& A, cudaStream_t s) {
   using T = TileOf<NDIM, PPM, SMALL>;
   using S = SmemT<T, R>;
   // opt in to more than 48 KiB of dynamic shared memory (idempotent)
@@ -93,7 +94,7 @@ static cudaError_t launch_tile(const StageArgs& A, cudaStream_t s, int hi) {
   unsigned nb[3] = {1, 1, 1};
   const int w[3] = {T::TX, T::TY, A.lz};
   for (int d = 0; d < NDIM; ++d)
-    nb[d] = (unsigned)(((d == NDIM - 1 ? hi - A.lo : A.g.n[d]) + w[d] - 1) / w[d]);
+    nb[d] = (unsigned)(((d == NDIM - 1 ? A.hi - A.lo : A.g.n[d]) + w[d] - 1) / w[d]);
   stage_kernel<STAGE, NDIM, R, GEN, PPM, SMALL>
       <<<dim3(nb[0], nb[1], nb[2]), T::NT, S::BYTES, s>>>(A);
   return cudaGetLastError();
@@ -107,15 +108,15 @@ static cudaError_t launch_nd(const StageArgs& A, cudaStream_t s, int b0, int b1)
   const int n = A.g.n[NDIM - 1], rows = (n + W - 1) / W;
   if (b1 < 0 || b1 > rows) b1 = rows;
   if (b0 < 0 || b0 >= b1) return cudaErrorInvalidValue;
-  const int hi = b1 * W < n ? b1 * W : n;
   StageArgs a = A;
   a.lo = b0 * W;
+  a.hi = b1 * W < n ? b1 * W : n;
   const TilePlan P = plan_tiles(A.g, MIXED, PPM, STAGE != 0);
   a.lz = P.lz;
   flux_weights(A.g, A.ph, MIXED, STAGE == 0 ? 1.0 : STAGE == 1 ? A.dt : 0.5 * A.dt, a.wE, a.wF);
   if constexpr (STAGE != 0)
-    if (P.small) return launch_tile<STAGE, NDIM, R, GEN, PPM, true>(a, s, hi);
-  return launch_tile<STAGE, NDIM, R, GEN, PPM, false>(a, s, hi);
+    if (P.small) return launch_tile<STAGE, NDIM, R, GEN, PPM, true>(a, s);
+  return launch_tile<STAGE, NDIM, R, GEN, PPM, false>(a, s);
 }
 
 template <int STAGE, typename R, bool GEN, bool PPM>

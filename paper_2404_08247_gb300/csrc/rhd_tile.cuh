@@ -34,9 +34,10 @@ struct TileT {
 
 // The tiles of the grid kernels (shapes and the planes a 3-D block marches
 // through: TilePlan, rhd_stage.cuh).  SMALL: one or two warps, for grids that
-// leave SMs idle with the large tile; rows a launch over part of a grid counts
-// in (the large tile's width along the slowest axis, 8 planes in 3-D) are
-// whole numbers of small ones.
+// leave SMs idle with the large tile.  A launch over part of a grid counts in
+// rows of kRowCells along the slowest axis (the large tile's width, 8 planes in
+// 3-D), each a whole number of tiles; a 3-D block marches up to 16 planes, but
+// never past the launch's end (block_planes).
 constexpr int kRowCells[4] = {0, 256, 8, 8};
 template <int NDIM, bool SMALL>
 struct TileShape;
