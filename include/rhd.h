@@ -128,6 +128,13 @@ typedef struct {
   int precision;       /* rhd_precision */
   double newton_rtol;  /* inner convergence tolerance (Sec. 3.3: 1e-13) */
   double outer_rtol;   /* outer convergence tolerance (Sec. 3.3: 1e-13) */
+  /* Both tests are applied to the iteration, whichever arithmetic its passes
+   * run in.  Where it runs on pairs of floats (constant chi, both tolerances
+   * 5e-14 or more), a last double-precision pass repeats its last one: it takes
+   * one Newton update, which removes the pairs' rounding from the residual (if
+   * that is within 1e4 newton_rtol), and accepts the outer stage within
+   * outer_rtol + min(outer_rtol, 1e-13), 1e-13 being the pairs' rounding; a cell
+   * that misses either goes on in double precision. */
   int newton_max_iter; /* bound on Newton updates per inner solve */
   int outer_max_iter;  /* bound on outer passes per local solve */
   /* -- added after the fields above; rhd_params_default sets them -- */

@@ -323,6 +323,7 @@ void rhd::fill_geometry(const rhd_params* p, Geometry& g, Physics& ph) {
   ph.hll_mode = p->hll_mode;
   ph.newton_rtol = p->newton_rtol;
   ph.outer_rtol = p->outer_rtol;
+  ph.outer_settle = p->outer_rtol + std::min(p->outer_rtol, 1e-13);
   ph.newton_max = p->newton_max_iter;
   ph.outer_max = p->outer_max_iter;
   ph.scheme = p->scheme;
