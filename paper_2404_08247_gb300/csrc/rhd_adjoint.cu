@@ -50,7 +50,7 @@ __device__ __forceinline__ long long face_index(const Geometry& g, int d, int x,
 __device__ __forceinline__ double half_slope_branch(double um, double u0, double up, int& br) {
   double dm = u0 - um, dp = up - u0;
   long long bm = dbits(dm), bp = dbits(dp);
-  long long am = bm & kMag, ap = bp & kMag, aq = quarter_bits(dm + dp);
+  long long am = bm & kMag, ap = bp & kMag, aq = quarter_mag(abs_bits(dm + dp));
   br = 0;
   if (!(((bm ^ bp) >= 0) & (am != 0) & (ap != 0))) return 0.0;
   long long m = min(min(am, ap), aq);

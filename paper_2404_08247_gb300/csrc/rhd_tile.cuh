@@ -602,10 +602,12 @@ __device__ __forceinline__ void stage_tile(const StageArgs& A, int x0, int y0, i
       cell_of<T, R>(ring + ((kbeg - 1) & 3) * S::PLANE, own, u0);
       cell_of<T, R>(ring + ((kbeg + 0) & 3) * S::PLANE, own, up);
       cell_of<T, R>(ring + ((kbeg + 1) & 3) * S::PLANE, own, upp);
+      R h[4];
+      half_slopes(um, u0, up, h);
+      half_slopes(u0, up, upp, hz);
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
-        hz[q] = half_slope(u0[q], up[q], upp[q]);
-        L[q] = u0[q] + half_slope(um[q], u0[q], up[q]);
+        L[q] = u0[q] + h[q];
         Rr[q] = up[q] - hz[q];
       }
     }
@@ -700,9 +702,9 @@ __device__ __forceinline__ void stage_tile(const StageArgs& A, int x0, int y0, i
         cell_of<T, R>(pl, own, u0);
         cell_of<T, R>(ring + ((k + 1) & 3) * S::PLANE, own, u1);
         cell_of<T, R>(ring + ((k + 2) & 3) * S::PLANE, own, u2);
+        half_slopes(u0, u1, u2, hz1);
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-          hz1[q] = half_slope(u0[q], u1[q], u2[q]);
           L[q] = u0[q] + hz[q];
           Rr[q] = u1[q] - hz1[q];
         }
@@ -721,8 +723,10 @@ __device__ __forceinline__ void stage_tile(const StageArgs& A, int x0, int y0, i
         cell_of<T, R>(pl, c - st, um);
         cell_of<T, R>(pl, c, u0);
         cell_of<T, R>(pl, c + st, up);
+        double h[4];
+        half_slopes(um, u0, up, h);
 #pragma unroll
-        for (int q = 0; q < 4; ++q) out[q * sn] = half_slope(um[q], u0[q], up[q]);
+        for (int q = 0; q < 4; ++q) out[q * sn] = h[q];
       };
       slope(own, 1, sx + ty * (TX + 2) + tx + 1, S::SX);
       if (NDIM >= 2) slope(own, S::PW, sy + (ty + 1) * TX + tx, S::SY);
@@ -831,10 +835,20 @@ __device__ __forceinline__ void stage_tile(const StageArgs& A, int x0, int y0, i
 #pragma unroll
         for (int q = 0; q < 8; ++q) y[q] = RHD_LD(A.st, A.yt[q], idx, g.ncell);
       } else if (STAGE == 2) {
+        bool tiny = false;
 #pragma unroll
-        for (int q = 0; q < 8; ++q)
-          y[q] = half_of(add(RHD_LD(A.st, A.yn[q], idx, g.ncell),
-                             RHD_LD(A.st, A.yt[q], idx, g.ncell)));
+        for (int q = 0; q < 8; ++q) {
+          const double sum = add(RHD_LD(A.st, A.yn[q], idx, g.ncell),
+                                 RHD_LD(A.st, A.yt[q], idx, g.ncell));
+          tiny = tiny || half_is_tiny(sum);
+          y[q] = half_or_zero(sum);
+        }
+        if (tiny) {  // a mean below the normal range
+#pragma unroll
+          for (int q = 0; q < 8; ++q)
+            y[q] = mul(0.5, add(RHD_LD(A.st, A.yn[q], idx, g.ncell),
+                                RHD_LD(A.st, A.yt[q], idx, g.ncell)));
+        }
       }
       // flux differences in double: the difference of two floats is exact in
       // double, so the update telescopes across cells in both precisions
