@@ -66,13 +66,11 @@ __device__ __forceinline__ Pair root(Pair a) {
   const float t = __fadd_rn(__fmaf_rn(-s, s, a.hi), a.lo);
   return {s, __fmul_rn(t, 0.5f * y)};
 }
-__device__ __forceinline__ Pair square(Pair a) { return a * a; }
-__device__ __forceinline__ float value(Pair a) { return a.hi; }
 
 // x 2^-s as a pair, by integer operations and one 32-bit conversion: hi is x
 // with its mantissa cut to 24 bits, lo the next 29 rounded to 24.  Below 2^-70
 // the pair is zero; false (and zero) where x 2^-s exceeds the float range or x
-// is not finite.
+// is not finite.  s > -953, so that a zero or subnormal x counts as below 2^-70.
 __device__ __forceinline__ bool split_scaled(double x, int s, Pair& p) {
   const long long b = __double_as_longlong(x);
   const int e = (int)((b >> 52) & 0x7ff) - s;  // biased exponent of x 2^-s
@@ -87,8 +85,8 @@ __device__ __forceinline__ bool split_scaled(double x, int s, Pair& p) {
   return true;
 }
 
-// hi + lo as a double times 2^s (a double addition; the widening by integer
-// operations, a float below the normal range counting as zero)
+// hi + lo as a double times 2^s, |s| <= 895 (a double addition; the widening by
+// integer operations, a float below the normal range counting as zero)
 __device__ __forceinline__ double widened(float f, int s) {
   const unsigned u = __float_as_uint(f);
   if ((u & 0x7f800000u) == 0u) return 0.0;

@@ -23,7 +23,11 @@ struct StartConsts {
   int ok;
 };
 
-inline PairScaled pair_scaled(double x, int& ok) {
+// emax: with it and the bound of 700 on E_tot's exponent the exponents that
+// pair_start scales by stay within split_scaled's and widened's ranges (the host
+// checks once what a test a cell would cost the mixed box 1.7 % for)
+constexpr int kUnitMax = 190;  // of chat and c/chat; 400 of the others
+inline PairScaled pair_scaled(double x, int& ok, int emax = 400) {
   PairScaled p = {{0.f, 0.f}, 0};
   if (!(x > 0.0) || !isfinite(x)) {
     ok = 0;
@@ -33,7 +37,7 @@ inline PairScaled pair_scaled(double x, int& ok) {
   p.e -= 1;
   p.m.hi = (float)m;
   p.m.lo = (float)(m - (double)p.m.hi);
-  if (p.e < -400 || p.e > 400) ok = 0;
+  if (p.e < -emax || p.e > emax) ok = 0;
   return p;
 }
 
@@ -43,11 +47,11 @@ inline void fill_start(StartConsts& K, double c, double chat, double a_rad, doub
   K.newton_rtol = (float)fmin(newton_rtol, 1e30);
   K.outer_rtol = (float)fmin(outer_rtol, 1e30);
   if (!(newton_rtol >= 5e-14 && outer_rtol >= 5e-14)) K.ok = 0;  // below the pairs' reach
-  K.inv_chat = pair_scaled(1.0 / chat, K.ok);
-  K.chat = pair_scaled(chat, K.ok);
+  K.inv_chat = pair_scaled(1.0 / chat, K.ok, kUnitMax);
+  K.chat = pair_scaled(chat, K.ok, kUnitMax);
   K.inv_c = pair_scaled(1.0 / c, K.ok);
-  K.chat_over_c = pair_scaled(chat / c, K.ok);
-  K.c_over_chat = pair_scaled(c / chat, K.ok);
+  K.chat_over_c = pair_scaled(chat / c, K.ok, kUnitMax);
+  K.c_over_chat = pair_scaled(c / chat, K.ok, kUnitMax);
   K.c2 = pair_scaled(c * c, K.ok);
   K.inv_c2 = pair_scaled(1.0 / (c * c), K.ok);
   K.q4 = pair_scaled(sqrt(sqrt(c / chat * a_rad)) / cv_spec, K.ok);
