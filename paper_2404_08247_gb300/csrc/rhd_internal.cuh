@@ -311,8 +311,10 @@ __device__ __forceinline__ double rsqrt_pos(double x) {
   const double y = rsqrt_seed(x);
   return fma(half_normal(y), fma(-mul(x, y), y, 1.0), y);
 }
+// (NaN for x = 0: the square of an E below 1e-162 vanishes, and a closure formed
+// from a root of zero would be a pressure of -E/3)
 __device__ __forceinline__ double sqrt_pos(double x) {
-  if (!seed_normal(x)) return sqrt(x);
+  if (!seed_normal(x)) return mul(x, 1.0 / sqrt(x));
   const double y = rsqrt_seed(x), t = mul(x, y);
   return fma(fma(-t, t, x), half_normal(y), t);
 }
@@ -556,8 +558,8 @@ __device__ __forceinline__ void face_side(int d, double q[4], int closure, doubl
     t = mul(x, y);
     h = fma(fma(-t, t, x), half_normal(y), t);
   } else {
-    t = h = sqrt(x);
-    y = 1.0 / h;
+    y = 1.0 / sqrt(x);
+    t = h = mul(x, y);  // NaN for x = 0, as sqrt_pos
   }
   if (over) {
     const double sc = mul(E, fma(half_normal(y), fma(-t, y, 1.0), y));
