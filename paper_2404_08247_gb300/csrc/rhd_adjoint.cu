@@ -392,7 +392,11 @@ __device__ __forceinline__ void gather_axis(const Geometry& g, const double* fp,
 // own block is al I plus products of v and Ft:
 //   d mu1 = x1 - (c/chat) x0 - (bv - (c/chat) a0) V - bu U,
 //   al mu = x - v (vv V + uv U - ev mu1) - Ft (vu V + uu U - eu mu1),
-// and its products with v and Ft are a 2 x 2 system for V and U.  All parts are
+// and its products with v and Ft are a 2 x 2 system for V and U.  The Jacobian's
+// determinant is d al det(2 x 2), and d, al > 0 for |v| < c (d = 1 + k g + (c/chat)
+// dR/dEgas; hb |Ft| <= 1, so al >= 1 + k (g - |v|/c)), so that the 2 x 2 system is
+// singular where the Jacobian is; it is scaled by a power of two near 1/al, or its
+// determinant, of order k^2, would overflow from k = 1e154 on.  All parts are
 // linear in these coefficients: 200 FP64 operations a cell, where the matrix
 // took 450; its m and F cotangents, in 64-bit terms, are the more accurate.
 // With the faces' optical-depth factors from the forward's arrays a 512^2
@@ -464,14 +468,16 @@ __device__ bool ls_adjoint(const Physics& ph, double tdt, double rho, double chi
   const double m0 = fma(-cr, x0, x1) * id, mV = -fma(cr, kB, bv) * id, mU = -bu * id;
   const double AV = fma(-ev, mV, vv), AU = fma(-ev, mU, uv), A0 = -ev * m0;
   const double BV = fma(-eu, mV, vu), BU = fma(-eu, mU, uu), B0 = -eu * m0;
-  const double M11 = fma(svv, AV, fma(svu, BV, al)), M12 = fma(svv, AU, svu * BU);
-  const double M21 = fma(svu, AV, suu * BV), M22 = fma(svu, AU, fma(suu, BU, al));
+  const long long ab = dbits(al) & kMag;
+  const double sc = __longlong_as_double((2046ll << 52) - (ab & kInfBits));
+  const double M11 = fma(svv, AV, fma(svu, BV, al)) * sc, M12 = fma(svv, AU, svu * BU) * sc;
+  const double M21 = fma(svu, AV, suu * BV) * sc, M22 = fma(svu, AU, fma(suu, BU, al)) * sc;
   const double r1 = fma(-svv, A0, fma(-svu, B0, dot3(v, x)));
   const double r2 = fma(-svu, A0, fma(-suu, B0, dot3(u, x)));
   const double det = fma(M11, M22, -M12 * M21);
-  const long long db = dbits(det) & kMag, ab = dbits(al) & kMag;
+  const long long db = dbits(det) & kMag;
   if (db == 0 || db >= kInfBits || ab == 0 || ab >= kInfBits) return false;
-  const double idet = copysign(rcp_pos(fabs(det)), det);
+  const double idet = copysign(rcp_pos(fabs(det)), det) * sc;
   const double V = fma(r1, M22, -M12 * r2) * idet, U = fma(M11, r2, -M21 * r1) * idet;
   const double m1 = fma(mV, V, fma(mU, U, m0));
   const double ca = fma(AV, V, fma(AU, U, A0)), cb = fma(BV, V, fma(BU, U, B0));
