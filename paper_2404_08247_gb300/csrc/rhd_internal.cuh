@@ -162,8 +162,8 @@ inline void slots_of(P* out, P base, int n) {
 //    together by integer operations.  2, 3 and 3 FP64 operations, where the
 //    series from the bare seed (2^-21) takes 3, 5 and 5 and two Newton steps 4,
 //    7 and 8; within 1 ulp.  Two steps of a 256^3 box 91.8 -> 87.8 ms, a 512^2
-//    gradient 38.5 -> 36.6, with PPM 17.7 -> 17.4.  The IEEE operation is used
-//    near the ends of the double range.
+//    gradient 38.5 -> 36.6, with PPM 17.7 -> 17.4.  Near the ends of the double
+//    range (2^-1018, 2^1017) IEEE operations are used, 1/sqrt in two roundings.
 constexpr long long kMag = 0x7fffffffffffffffll;
 constexpr long long kInfBits = 0x7ff0000000000000ll;
 
@@ -311,10 +311,14 @@ __device__ __forceinline__ double rsqrt_pos(double x) {
   const double y = rsqrt_seed(x);
   return fma(half_normal(y), fma(-mul(x, y), y, 1.0), y);
 }
-// (NaN for x = 0: the square of an E below 1e-162 vanishes, and a closure formed
-// from a root of zero would be a pressure of -E/3)
+// Outside the seeds' range: sqrt, but NaN for x = 0 (the square of an E below
+// 1e-162 vanishes, and a closure formed from a root of zero would be a pressure of
+// -E/3).
+__device__ __forceinline__ double sqrt_or_nan(double x) {
+  return dbits(x) == 0 ? __longlong_as_double(0x7ff8000000000000ll) : sqrt(x);
+}
 __device__ __forceinline__ double sqrt_pos(double x) {
-  if (!seed_normal(x)) return mul(x, 1.0 / sqrt(x));
+  if (!seed_normal(x)) return sqrt_or_nan(x);
   const double y = rsqrt_seed(x), t = mul(x, y);
   return fma(fma(-t, t, x), half_normal(y), t);
 }
@@ -558,8 +562,8 @@ __device__ __forceinline__ void face_side(int d, double q[4], int closure, doubl
     t = mul(x, y);
     h = fma(fma(-t, t, x), half_normal(y), t);
   } else {
-    y = 1.0 / sqrt(x);
-    t = h = mul(x, y);  // NaN for x = 0, as sqrt_pos
+    t = h = sqrt_or_nan(x);
+    y = 1.0 / h;
   }
   if (over) {
     const double sc = mul(E, fma(half_normal(y), fma(-t, y, 1.0), y));
