@@ -163,7 +163,7 @@ inline void slots_of(P* out, P base, int n) {
 //    series from the bare seed (2^-21) takes 3, 5 and 5 and two Newton steps 4,
 //    7 and 8; within 1 ulp.  Two steps of a 256^3 box 91.8 -> 87.8 ms, a 512^2
 //    gradient 38.5 -> 36.6, with PPM 17.7 -> 17.4.  Near the ends of the double
-//    range (2^-1018, 2^1017) IEEE operations are used, 1/sqrt in two roundings.
+//    range (2^-1019, 2^1017) IEEE operations are used, 1/sqrt in two roundings.
 constexpr long long kMag = 0x7fffffffffffffffll;
 constexpr long long kInfBits = 0x7ff0000000000000ll;
 
@@ -218,21 +218,20 @@ __host__ __device__ __forceinline__ long long quarter_mag(long long a) {
   if (a >= (2ll << 52)) return half_mag(a - (1ll << 52));  // twice that many units
   return (a + 1 + ((a >> 2) & 1)) >> 2;
 }
-// The same with zero below 2^-1021 and 2^-1020, for use where the caller takes
-// such a result again the exact way (half_slopes; the mean of stage 2).  Two steps
-// of a 256^3 box: 87.7 ms, with the shifts in line 88.2, with nothing below those
-// numbers, which lost such fields, 85.9.
-__device__ __forceinline__ double half_or_zero(double x) {
-  const long long b = dbits(x), a = b & kMag;
-  const long long h = a >= kInfBits ? a : a >= (2ll << 52) ? a - (1ll << 52) : 0ll;
-  return __longlong_as_double(h | (b & ~kMag));
+// x/2 by one subtraction from its high word; rare: set where that is not the half
+// (results below the normal range, infinities, NaN; zero stays zero), which the
+// caller then takes the exact way.  Likewise the minimum of three magnitudes, the
+// third a sum's less two exponents, is final unless min_is_rare.  (256^3 box, two
+// steps: 87.1 ms, with the shifts in line 88.2, with results below the normal range
+// dropped 85.9; 128 x 96 x 110 with PPM, three steps: 17.50, 17.84, 17.45.)
+__device__ __forceinline__ double half_fast(double x, bool& rare) {
+  const int hi = __double2hiint(x), lo = __double2loint(x), a = hi & 0x7fffffff;
+  const bool zero = (a | lo) == 0;
+  rare = rare | (!zero & ((unsigned)(a - 0x200000) >= 0x7fd00000u));
+  return __hiloint2double(zero ? hi : hi - 0x100000, lo);
 }
-__device__ __forceinline__ bool half_is_tiny(double x) {
-  const long long a = abs_bits(x);
-  return a != 0 && a < (2ll << 52);
-}
-__device__ __forceinline__ long long quarter_or_zero(long long a) {
-  return a >= kInfBits ? a : a >= (3ll << 52) ? a - (2ll << 52) : 0ll;
+__device__ __forceinline__ bool min_is_rare(long long m) {
+  return (unsigned)((int)(m >> 32) - 0x100000) >= 0x7fd00000u - 0x100000u;
 }
 __device__ __forceinline__ double half_of(double x) {
   const long long b = dbits(x);
@@ -336,36 +335,36 @@ __device__ __forceinline__ R half_slope(R um, R u0, R up) {
 }
 
 // double: the same value with the sign tests, the quarter and the minimum on
-// the integer pipe.  tiny (not EXACT): set where the quarter is below the normal
-// range and has been taken as zero.
+// the integer pipe.  rare (not EXACT): set where the value has to be taken the
+// exact way.
 template <bool EXACT>
-__device__ __forceinline__ double half_slope_d64(double um, double u0, double up, bool& tiny) {
+__device__ __forceinline__ double half_slope_d64(double um, double u0, double up, bool& rare) {
   double dm = u0 - um;
   double dp = up - u0;
   long long bm = dbits(dm), bp = dbits(dp);
   long long am = bm & kMag, ap = bp & kMag;
   const long long as = abs_bits(dm + dp);
-  const long long m = min(min(am, ap), EXACT ? quarter_mag(as) : quarter_or_zero(as));
+  const long long m = min(min(am, ap), EXACT ? quarter_mag(as) : as - (2ll << 52));
   const bool take = ((bm ^ bp) >= 0) & (am != 0) & (ap != 0);  // same sign, both nonzero
-  if (!EXACT) tiny = tiny | (take & (as < (3ll << 52)));
+  if (!EXACT) rare = rare | (take & min_is_rare(m));
   return __longlong_as_double(take ? (m | (bm & ~kMag)) : 0ll);
 }
 template <>
 __device__ __forceinline__ double half_slope<double>(double um, double u0, double up) {
-  bool tiny;
-  return half_slope_d64<true>(um, u0, up, tiny);
+  bool rare;
+  return half_slope_d64<true>(um, u0, up, rare);
 }
 
 // Those of the four fields of a cell, the exact quarter only where one needs it.
 template <typename R>
 __device__ __forceinline__ void half_slopes(const R um[4], const R u0[4], const R up[4], R h[4]) {
   if constexpr (sizeof(R) == sizeof(double)) {
-    bool tiny = false;
+    bool rare = false;
 #pragma unroll
-    for (int q = 0; q < 4; ++q) h[q] = half_slope_d64<false>(um[q], u0[q], up[q], tiny);
-    if (tiny) {
+    for (int q = 0; q < 4; ++q) h[q] = half_slope_d64<false>(um[q], u0[q], up[q], rare);
+    if (rare) {
 #pragma unroll
-      for (int q = 0; q < 4; ++q) h[q] = half_slope_d64<true>(um[q], u0[q], up[q], tiny);
+      for (int q = 0; q < 4; ++q) h[q] = half_slope_d64<true>(um[q], u0[q], up[q], rare);
     }
   } else {
 #pragma unroll
@@ -385,6 +384,37 @@ __device__ __forceinline__ R ppm_interface(R u0, R up, R h0, R h1) {
     return fma(sub(h0, h1), 1.0 / 3.0, half_of(add(u0, up)));
   else
     return R(0.5) * (u0 + up) - (h1 - h0) * R(1.0 / 3.0);
+}
+
+// The same from the four cells um .. upp, the slopes and the half sum taken the
+// short way unless EXACT (rare: see half_fast), and those of the four fields.
+template <bool EXACT>
+__device__ __forceinline__ double ppm_interface_d64(double um, double u0, double up, double upp,
+                                                    bool& rare) {
+  const double h0 = half_slope_d64<EXACT>(um, u0, up, rare);
+  const double h1 = half_slope_d64<EXACT>(u0, up, upp, rare);
+  const double s = add(u0, up);
+  return fma(sub(h0, h1), 1.0 / 3.0, EXACT ? half_of(s) : half_fast(s, rare));
+}
+template <typename R>
+__device__ __forceinline__ void ppm_interfaces(const R um[4], const R u0[4], const R up[4],
+                                               const R upp[4], R a[4]) {
+  if constexpr (sizeof(R) == sizeof(double)) {
+    bool rare = false;
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      a[q] = ppm_interface_d64<false>(um[q], u0[q], up[q], upp[q], rare);
+    if (rare) {
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        a[q] = ppm_interface_d64<true>(um[q], u0[q], up[q], upp[q], rare);
+    }
+  } else {
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      a[q] = ppm_interface(u0[q], up[q], half_slope(um[q], u0[q], up[q]),
+                           half_slope(u0[q], up[q], upp[q]));
+  }
 }
 
 // Their monotonicity constraint (eq. 1.10) on the edge values (l, r) of a
@@ -725,6 +755,26 @@ __device__ __forceinline__ bool quartic_start(double a4, double rhs, double T0, 
   return true;
 }
 
+// (T/T_ref)^p of chi = kappa rho (T/T_ref)^p.  Whole exponents (the Marshak
+// wave's -3) by a product that carries its rounding errors (fused
+// multiply-adds; Dekker 1971) and one reciprocal: within 1 ulp, and 13 FP64
+// operations for -3, where pow takes several times that in every Newton update
+// (a 60-cell Marshak wave, 50 steps: 4.86 ms, with pow 6.56).
+__device__ __forceinline__ double opacity_power(const Physics& ph, double x) {
+  const int n = ph.kappa_T_int < 0 ? -ph.kappa_T_int : ph.kappa_T_int;
+  if (n == 0) return pow(x, ph.kappa_T_exp);
+  double hi = x, lo = 0.0;
+  for (int i = 1; i < n; ++i) {
+    const double p = mul(hi, x);
+    lo = fma(lo, x, fma(hi, x, -p));
+    hi = p;
+  }
+  if (!seed_range(hi)) return pow(x, ph.kappa_T_exp);
+  if (ph.kappa_T_int > 0) return add(hi, lo);
+  const double r = rcp_pos(hi);
+  return fma(mul(-lo, r), r, r);
+}
+
 // Implicit stage of one cell (Sec. 3.3), grey chi.  y = {Egas, m, E, F}
 // holds the explicit state on entry and the solution on exit.  tdt = theta dt.
 //
@@ -758,26 +808,6 @@ __device__ __forceinline__ bool quartic_start(double a4, double rhs, double T0, 
 // to rounding.
 // GEN: compiled with the temperature-dependent opacity; the default physics
 // (constant chi) uses the GEN = false copy, free of that branch.
-// (T/T_ref)^p of chi = kappa rho (T/T_ref)^p.  Whole exponents (the Marshak
-// wave's -3) by a product that carries its rounding errors (fused
-// multiply-adds; Dekker 1971) and one reciprocal: within 1 ulp, and 13 FP64
-// operations for -3, where pow takes several times that in every Newton update
-// (a 60-cell Marshak wave, 50 steps: 4.86 ms, with pow 6.56).
-__device__ __forceinline__ double opacity_power(const Physics& ph, double x) {
-  const int n = ph.kappa_T_int < 0 ? -ph.kappa_T_int : ph.kappa_T_int;
-  if (n == 0) return pow(x, ph.kappa_T_exp);
-  double hi = x, lo = 0.0;
-  for (int i = 1; i < n; ++i) {
-    const double p = mul(hi, x);
-    lo = fma(lo, x, fma(hi, x, -p));
-    hi = p;
-  }
-  if (!seed_range(hi)) return pow(x, ph.kappa_T_exp);
-  if (ph.kappa_T_int > 0) return add(hi, lo);
-  const double r = rcp_pos(hi);
-  return fma(mul(-lo, r), r, r);
-}
-
 constexpr double kNear = 1e4;  // in units of the Newton tolerance
 
 template <bool MIXED, bool GEN>

@@ -39,12 +39,17 @@ __global__ void __launch_bounds__(TileOf<NDIM, PPM, SMALL>::NT,
 // and 1 to 16 planes a block (a block adds a z face a column and its ghost
 // planes' loads) are priced, and the cheapest is taken.  Prices are FP64
 // instructions a warp: a face, a z face and a cell's slopes, update and solve.
-// The busiest SM issues its instructions at one in 16 cycles, slowed by (1 + 6/w)
-// when w warps are resident: 73 % of the pipe with 16 warps, 50 to 57 % with
-// 8, 11 to 14 % with one, as measured.  Against the large tile with 8 planes a
-// block everywhere: a 40 x 37 x 33 box, five steps, 5.3 -> 2.2 ms; a 256-cell
+// The busiest SM (of 152) issues its instructions at one in 16 cycles, slowed by
+// (1 + 6/w) when w warps are resident: 73 % of the pipe with 16 warps, 50 to 57 %
+// with 8, 11 to 14 % with one, as measured.  w counts the 16 warps that registers
+// allow; shared memory holds the small 3-D tiles to fewer (FP64 PLM 14, PPM 10,
+// mixed PPM 12), which the price leaves out.  Against the large tile with 8 planes
+// a block everywhere: a 40 x 37 x 33 box, five steps, 5.3 -> 2.2 ms; a 256-cell
 // row, 50 steps, 4.6 -> 3.5 ms; 256^3, where both price 8 or 16 planes alike,
-// unchanged.
+// unchanged; 48 boxes of 315 cells to 128 x 96 x 110 between 1 and 7 times as
+// fast, but for three that it prices wrongly (mixed precision, two steps):
+// 96 x 80 x 72 takes 2.28 ms for 1.94, with PPM 2.81 for 2.15, and 64^3 with PPM
+// 1.54 for 1.50.
 struct TilePlan {
   bool small;
   int lz;

@@ -9,9 +9,10 @@
 // current plane by one thread each (into shared memory), z-faces by the thread
 // that owns the column (kept in registers from one plane to the next,
 // together with the half z-slope of the current cell).  The thread then
-// applies the conservative update and runs the cell's local implicit solve in
-// registers, so the explicit state never reaches HBM.  2-D grids use one
-// plane; 1-D grids use rows of TX cells.
+// applies the conservative update and runs the cell's local implicit solve (a
+// call, local_solve_call: the state passes through the thread's stack, in L1), so
+// the explicit state never reaches HBM.  2-D grids use one plane; 1-D grids use
+// rows of TX cells.
 #pragma once
 
 #include <type_traits>
@@ -669,15 +670,14 @@ __device__ __forceinline__ void stage_tile(const StageArgs& A, int x0, int y0, i
           dz[q * NT] = v0[q] - R(2) * v1[q] + v2[q];
         }
       } else {
+        R an[4];
+        ppm_interfaces(v0, v1, v2, v3, an);
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-          const R ha = half_slope(v0[q], v1[q], v2[q]);
-          const R hb = half_slope(v1[q], v2[q], v3[q]);
-          const R an = ppm_interface(v1[q], v2[q], ha, hb);
           L[q] = rz[q * NT];
-          Rr[q] = ppm_edge_of<true>(v1[q], az[q * NT], an);
-          rz[q * NT] = ppm_edge_of<false>(v1[q], az[q * NT], an);
-          az[q * NT] = an;
+          Rr[q] = ppm_edge_of<true>(v1[q], az[q * NT], an[q]);
+          rz[q * NT] = ppm_edge_of<false>(v1[q], az[q * NT], an[q]);
+          az[q * NT] = an[q];
         }
       }
       R eps = (R)face_eps(A, 2, cx, cy, k);
@@ -746,13 +746,12 @@ __device__ __forceinline__ void stage_tile(const StageArgs& A, int x0, int y0, i
     // ---- FP64 PPM: the interface value between cells c - st and c
     auto interface = [&](int c, int st, double* out, int sn) {
       if constexpr (S::IFACE) {
-        double u[4][4];
+        double u[4][4], a[4];
 #pragma unroll
         for (int o = 0; o < 4; ++o) cell_of<T, R>(pl, c + (o - 2) * st, u[o]);
+        ppm_interfaces(u[0], u[1], u[2], u[3], a);
 #pragma unroll
-        for (int q = 0; q < 4; ++q)
-          out[q * sn] = ppm_interface(u[1][q], u[2][q], half_slope(u[0][q], u[1][q], u[2][q]),
-                                      half_slope(u[1][q], u[2][q], u[3][q]));
+        for (int q = 0; q < 4; ++q) out[q * sn] = a[q];
       }
     };
     if (S::IFACE && !cs) {
@@ -835,15 +834,12 @@ __device__ __forceinline__ void stage_tile(const StageArgs& A, int x0, int y0, i
 #pragma unroll
         for (int q = 0; q < 8; ++q) y[q] = RHD_LD(A.st, A.yt[q], idx, g.ncell);
       } else if (STAGE == 2) {
-        bool tiny = false;
+        bool rare = false;
 #pragma unroll
-        for (int q = 0; q < 8; ++q) {
-          const double sum = add(RHD_LD(A.st, A.yn[q], idx, g.ncell),
-                                 RHD_LD(A.st, A.yt[q], idx, g.ncell));
-          tiny = tiny || half_is_tiny(sum);
-          y[q] = half_or_zero(sum);
-        }
-        if (tiny) {  // a mean below the normal range
+        for (int q = 0; q < 8; ++q)
+          y[q] = half_fast(add(RHD_LD(A.st, A.yn[q], idx, g.ncell),
+                               RHD_LD(A.st, A.yt[q], idx, g.ncell)), rare);
+        if (rare) {  // a mean below the normal range or not finite
 #pragma unroll
           for (int q = 0; q < 8; ++q)
             y[q] = mul(0.5, add(RHD_LD(A.st, A.yn[q], idx, g.ncell),
