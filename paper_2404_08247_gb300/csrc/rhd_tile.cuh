@@ -671,7 +671,7 @@ __device__ __forceinline__ void stage_tile(const StageArgs& A, int x0, int y0, i
         }
       } else {
         R an[4];
-        ppm_interfaces(v0, v1, v2, v3, an);
+        ppm_interfaces<STAGE != 0>(v0, v1, v2, v3, an);
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
           L[q] = rz[q * NT];
@@ -749,7 +749,7 @@ __device__ __forceinline__ void stage_tile(const StageArgs& A, int x0, int y0, i
         double u[4][4], a[4];
 #pragma unroll
         for (int o = 0; o < 4; ++o) cell_of<T, R>(pl, c + (o - 2) * st, u[o]);
-        ppm_interfaces(u[0], u[1], u[2], u[3], a);
+        ppm_interfaces<STAGE != 0>(u[0], u[1], u[2], u[3], a);
 #pragma unroll
         for (int q = 0; q < 4; ++q) out[q * sn] = a[q];
       }

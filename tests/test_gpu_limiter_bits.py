@@ -30,7 +30,7 @@ __global__ void limiter_kernel(const double* u, int n, double* out) {
   for (int o = 0; o < 4; ++o)
     for (int q = 0; q < 4; ++q) c[o][q] = u[(o * 4 + q) * n + i];
   half_slopes(c[0], c[1], c[2], h);
-  ppm_interfaces(c[0], c[1], c[2], c[3], a);
+  ppm_interfaces<true>(c[0], c[1], c[2], c[3], a);
   for (int q = 0; q < 4; ++q) {
     const double s = __dadd_rn(c[1][q], c[2][q]), half = __dmul_rn(0.5, s);
     bool rare = false;
