@@ -54,7 +54,7 @@ template <>
 struct TileShape<2, true> { static constexpr int TX = 16, TY = 4; };
 template <>
 struct TileShape<1, true> { static constexpr int TX = 32, TY = 1; };
-// PPM tiles: the same shapes with the wider halo (3-D, FP64, large: 86 KB of
+// PPM tiles: the same shapes with the wider halo (3-D, FP64, large: 111 KB of
 // shared memory, two blocks per SM)
 template <int NDIM, bool PPM, bool SMALL>
 using TileOf = TileT<NDIM, TileShape<NDIM, SMALL>::TX, TileShape<NDIM, SMALL>::TY, PPM>;
